@@ -106,6 +106,7 @@ struct helm_dd {
     int64_t ct_sz = 0;
     std::vector<double2> slab_cy;
     int slab_ld = 0;
+    void* d_slab_scratch = nullptr;   // step vectors and partial sums of the 3-D strip solve
     size_t esize = 16;
     bool factored = false;
     bool prepared = false;
@@ -601,8 +602,8 @@ helm_status factor_slabs(helm_dd* h) {
         set_strip_io(h, s, (int)jj);
         const int n = s.W * Nz;
         s.nj = 0;
-        s.ld = (n + 3) & ~3;   // rows start 32-byte aligned, columns n.. zero
-        s.bs = (int64_t)n * s.ld;
+        s.ld = (n + 3) & ~3;   // row stride of the strip right-hand sides and solutions
+        s.bs = (int64_t)((n + 63) / 64) * 64 * n;   // tile layout (slab_ops.cuh)
         s.fac = fac;
         s.red = 0;
         s.xf = 0;
@@ -646,6 +647,9 @@ helm_status factor_slabs(helm_dd* h) {
         CK(h, cudaMemcpy(h->d_slab_sxz, f.data(), f.size() * sizeof(double2), cudaMemcpyHostToDevice));
     }
     h->slab_ld = ldmax;
+    if (h->d_slab_scratch) cudaFree(h->d_slab_scratch);
+    h->d_slab_scratch = nullptr;
+    CK(h, cudaMalloc(&h->d_slab_scratch, slab_sweep_scratch(nmax, h->esize)));
     CK(h, cudaMemcpyAsync(h->d_strips, h->strips.data(), h->strips.size() * sizeof(StripDev),
                           cudaMemcpyHostToDevice, h->stream));
     CK(h, cudaMemsetAsync(h->d_status, 0, sizeof(int), h->stream));
@@ -1119,7 +1123,7 @@ helm_status run_precond_slabs(helm_dd* h, const double2* in, double2* out, int B
     auto solve = [&](int j, const SweepStep& sp, int slot) -> cudaError_t {
         SlabWork wk{rbuf, ybuf[slot], sp.prev >= 0 ? ybuf[slot ^ 1] : nullptr,
                     (const char*)h->d_slab_sxz + h->slab_sxz_off[j] * (int64_t)h->esize, h->ct_sz,
-                    h->slab_cy.data(), ld, B, (unsigned*)bf.counters, h->d_status};
+                    h->slab_cy.data(), ld, B, h->d_slab_scratch, (unsigned*)bf.counters, h->d_status};
         const StripDev* pst = sp.prev >= 0 ? &h->strips[sp.prev] : nullptr;
         if (mixed) return launch_slab_solve<float2>(h->geom, h->strips[j], pst, sp, wk, h->d_pool[0], h->stream, &h->timer);
         return launch_slab_solve<double2>(h->geom, h->strips[j], pst, sp, wk, h->d_pool[0], h->stream, &h->timer);
@@ -1589,7 +1593,7 @@ helm_status run_local_solves(helm_dd* h, const double2* F, double2* Ut, int B, c
         for (int j = 0; j < J; ++j) {
             const SweepStep sp = step_of(j);
             SlabWork wk{rbuf, ybuf, nullptr, (const char*)h->d_slab_sxz + h->slab_sxz_off[j] * (int64_t)h->esize,
-                        h->ct_sz, h->slab_cy.data(), ld, B, (unsigned*)bf.counters, h->d_status};
+                        h->ct_sz, h->slab_cy.data(), ld, B, h->d_slab_scratch, (unsigned*)bf.counters, h->d_status};
             cudaError_t e = mixed ? launch_slab_solve<float2>(h->geom, h->strips[j], nullptr, sp, wk, h->d_pool[0],
                                                               h->stream, &h->timer)
                                   : launch_slab_solve<double2>(h->geom, h->strips[j], nullptr, sp, wk, h->d_pool[0],
@@ -2101,6 +2105,7 @@ void helm_dd_destroy(helm_dd* h) {
     for (auto p : h->d_pool) cudaFree(p);
     cudaFree(h->d_ct);
     cudaFree(h->d_slab_sxz);
+    cudaFree(h->d_slab_scratch);
     cudaFree(h->d_counters);
     cudaFree(h->d_icols);
     cudaFree(h->d_rab);

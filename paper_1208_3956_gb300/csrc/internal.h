@@ -176,21 +176,18 @@ struct SlabWork {
     const double2* cy_host;   // host: -alpha_y(y_{k-1/2}) / h^2, k = 0 .. Ny
     int ld;                   // row stride of rbuf / ybuf / pybuf (>= every strip's n)
     int B;
-    unsigned* bar;            // grid-barrier counter of the strip-solve kernel
+    void* scratch;            // slab_sweep_scratch bytes: the strip solve's step vectors and partial sums
+    unsigned* bar;            // counters of the strip-solve kernel (16 KB)
     int* status;              // error word (7 = a bounded wait gave up)
 };
-// Factor blocks X_k = S_k^{-1} of strip st into pool + st.fac (row-major, leading
-// dimension st.ld, st.bs elements per block), k = 0 .. Ny-1.
+size_t slab_sweep_scratch(int nmax, size_t esize);
+// Factor blocks X_k = S_k^{-1} of strip st into pool + st.fac (tile layout of slab_ops.cuh,
+// st.bs elements per block), k = 0 .. Ny-1.
 template <typename C>
 cudaError_t launch_slab_factor(const Geom& g, const StripDev& st, void* pool, const SlabScratch& sc, int* status,
                                cudaStream_t s, KernelTimer* tm);
-// M (column-major, leading dimension ldm) = D_k - C_k Xp C_k (Xp = X_{k-1} in the sweep
-// layout, leading dimension ld; M = D_k when Xp is null).
-template <typename C>
-cudaError_t launch_slab_build(const Geom& g, const StripDev& st, int k, const C* Xp, int ld, C* M, int ldm,
-                              cudaStream_t s, KernelTimer* tm);
-// slab_tc.cu: the blocks X_k = S_k^{-1}, k = 0 .. Ny-1, of up to 8 strips side by side in
-// complex64, inverted by blocked Gauss-Jordan elimination whose rank-12 updates run on the
+// slab_tc.cu: the blocks X_k = S_k^{-1}, k = 0 .. Ny-1, of up to 8 strips (16 chains) side by
+// side in complex64, inverted by blocked Gauss-Jordan elimination whose updates run on the
 // tensor cores; scratch of slab_factor_tc_scratch(max n, strips) bytes.
 size_t slab_factor_tc_scratch(int nmax, int ns);
 cudaError_t launch_slab_factor_tc(const Geom& g, const StripDev* strips, int ns, void* pool, void* scratch,

@@ -11,21 +11,26 @@
 //   C_k(e)       = -s_x(c) s_z(z) a_y(k-1/2) / h^2      (couples rows k-1, k)
 // with s = 1/alpha at integer points and a = alpha at half points.
 //
-// Factorisation (Algorithm 1, top down): X_k = S_k^{-1},
-//   S_0 = D_0,  S_k = D_k - C_k X_{k-1} C_k,
-// each S_k inverted by Gauss-Jordan elimination with partial (row) pivoting on
-// the whole GPU (one cooperative launch per block).  Solve of a strip
-// (block forward and back substitution):
-//   y_k = X_k (r_k - C_k y_{k-1}),   k = 0 .. N_y-1
-//   x_k = y_k - X_k C_{k+1} x_{k+1}, k = N_y-2 .. 0
-// all 2 N_y - 1 steps in one cooperative launch (k_slab_sweep), each a
-// matrix-vector product that streams X_k from HBM through shared memory.
+// Factorisation (Algorithm 1) from both ends toward a middle row t = (N_y-1)/2, so that the
+// elimination and the solves are two independent chains: X_k = S_k^{-1},
+//   k < t:  S_k = D_k - C_k X_{k-1} C_k              (top down)
+//   k > t:  S_k = D_k - C_{k+1} X_{k+1} C_{k+1}      (bottom up)
+//   S_t = D_t - C_t X_{t-1} C_t - C_{t+1} X_{t+1} C_{t+1}
+// each S_k inverted by Gauss-Jordan elimination with partial (row) pivoting: complex64 on the
+// tensor cores, the rows of both chains of several strips side by side (slab_tc.cu), complex128
+// on the whole GPU (one cooperative launch per block).  Solve of a strip (block elimination
+// toward t and substitution outward):
+//   y_k = X_k (r_k - C_k y_{k-1}),      k < t;    y_k = X_k (r_k - C_{k+1} y_{k+1}),  k > t
+//   x_t = X_t (r_t - C_t y_{t-1} - C_{t+1} y_{t+1})
+//   x_k = y_k - X_k C_{k+1} x_{k+1},    k < t;    x_k = y_k - X_k C_k x_{k-1},        k > t
+// all 2 N_y - 1 block steps in one cooperative launch (k_slab_sweep), each a matrix product
+// with the right-hand sides' vectors that streams X_k from HBM through shared memory.
 #include <algorithm>
 
 #include <type_traits>
 
 #include "common.cuh"
-#include "strip_ops.cuh"
+#include "slab_ops.cuh"
 #include "internal.h"
 
 namespace helm {
@@ -62,84 +67,17 @@ __device__ __forceinline__ void add_release(unsigned* ctr) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr) : "memory");
 }
 
-// ------------------------------------------------------------ block entries
-__device__ __forceinline__ double2 slab_sz(const Geom& g, int z) { return cinv(g.gz_int[z]); }
-
-__device__ double2 slab_diag(const Geom& g, const StripDev& st, int k, int c, int z) {
-    const double2 sx = strip_sx(g, st, c), sy = glob_sy(g, k), sz = slab_sz(g, z);
-    const double2 xs = cadd(strip_ax_half(g, st, c + 1), strip_ax_half(g, st, c));
-    const double2 ys = cadd(g.gy_half[k + 1], g.gy_half[k]);
-    const double2 zs = cadd(g.gz_half[z + 1], g.gz_half[z]);
-    double2 d = cadd(cadd(cmul(cmul(sy, sz), xs), cmul(cmul(sx, sz), ys)), cmul(cmul(sx, sy), zs));
-    d = cscale(d, g.inv_h2);
-    const double k2 = g.k2[((int64_t)z * g.Ny + k) * g.Nx + strip_k2_col(st, c)];
-    return csub(d, cscale(cmul(cmul(sx, sy), sz), k2));
-}
-// entry (e, e+1), e = z W + c, c + 1 < W
-__device__ double2 slab_xoff(const Geom& g, const StripDev& st, int k, int c, int z) {
-    return cscale(cmul(cmul(glob_sy(g, k), slab_sz(g, z)), strip_ax_half(g, st, c + 1)), -g.inv_h2);
-}
-// entry (e, e+W), z + 1 < N_z
-__device__ double2 slab_zoff(const Geom& g, const StripDev& st, int k, int c, int z) {
-    return cscale(cmul(cmul(strip_sx(g, st, c), glob_sy(g, k)), g.gz_half[z + 1]), -g.inv_h2);
-}
-// D_k(r, a) for any pair (zero off the stencil)
-__device__ double2 slab_dentry(const Geom& g, const StripDev& st, int k, int r, int a) {
-    const int W = st.W;
-    const int lo = imin(r, a), d = r > a ? r - a : a - r;
-    if (d != 0 && d != 1 && d != W) return make_double2(0.0, 0.0);
-    const int c = lo % W, z = lo / W;
-    if (d == 0) return slab_diag(g, st, k, c, z);
-    if (d == 1 && c + 1 < W) return slab_xoff(g, st, k, c, z);
-    if (d == W) return slab_zoff(g, st, k, c, z);
-    return make_double2(0.0, 0.0);
-}
-
-// M (column-major, ldm) = - C_k Xp C_k, Xp = X_{k-1} in the row-major sweep layout
-// (leading dimension ld), or M = 0 for k = 0; k_slab_dadd then adds D_k.  32 x 32 tiles.
+// M (column-major, ldm) = - C_k Xp C_k - C_{k+1} Xn C_{k+1}, Xp = X_{k-1} and Xn = X_{k+1} in the
+// tile layout (null: no such term); k_slab_dadd then adds D_k.
 template <typename C>
-__global__ void __launch_bounds__(256) k_slab_build(Geom g, StripDev st, int k, const C* __restrict__ Xp, int ld,
-                                                    C* __restrict__ M, int ldm) {
-    __shared__ C tile[32][33];
-    __shared__ C cr[32], cc[32];
-    const int n = st.W * g.Nz;
-    const int r0 = blockIdx.y * 32, a0 = blockIdx.x * 32;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 8 rows of 32
-    if (Xp) {
-        for (int i = ty; i < 32; i += 8) {
-            const int r = r0 + i, a = a0 + tx;
-            tile[i][tx] = (r < n && a < n) ? Xp[(int64_t)r * ld + a] : CT<C>::zero();
-        }
-        if (threadIdx.x < 64) {
-            const int e = (threadIdx.x < 32 ? r0 : a0) + tx;
-            // C_k(e) = s_x(c) s_z(z) (-alpha_y(y_{k-1/2}) / h^2) from the working-precision table
-            const C* ct = reinterpret_cast<const C*>(g.ct);
-            const C v = e < n ? cmul(cmul(ct[st.ctab + e % st.W], ct[g.ct_sz + e / st.W]), ct[g.ct_cy + k])
-                              : CT<C>::zero();
-            (threadIdx.x < 32 ? cr : cc)[tx] = v;
-        }
-    }
-    __syncthreads();
-    // write column a0+i, rows r0+tx (coalesced along rows)
-    for (int i = ty; i < 32; i += 8) {
-        const int a = a0 + i, r = r0 + tx;
-        if (a >= n || r >= n) continue;
-        M[(int64_t)a * ldm + r] = Xp ? cneg(cmul(cmul(cr[tx], tile[tx][i]), cc[i])) : CT<C>::zero();
-    }
+__global__ void __launch_bounds__(256) k_slab_build(Geom g, StripDev st, int k, const C* __restrict__ Xp,
+                                                    const C* __restrict__ Xn, C* __restrict__ M, int ldm) {
+    slab_build_entries<C>(g, st, k, Xp, Xn, M, ldm);
 }
 
-// M(r, a) += D_k(r, a) on the stencil entries of row r: a = r, r +- 1 (same z), r +- W; one
-// entry per thread (the entries are evaluated in FP64, so they are spread over the GPU).
 template <typename C>
 __global__ void __launch_bounds__(64) k_slab_dadd(Geom g, StripDev st, int k, C* __restrict__ M, int ldm) {
-    const int n = st.W * g.Nz, W = st.W;
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < 5 * n; e += gridDim.x * blockDim.x) {
-        const int r = e / 5, i = e % 5, c = r % W;
-        const int a = i == 0 ? r : i == 1 ? (c > 0 ? r - 1 : -1) : i == 2 ? (c + 1 < W ? r + 1 : -1) : i == 3 ? r - W : r + W;
-        if (a < 0 || a >= n) continue;
-        C* p = M + (int64_t)a * ldm + r;
-        *p = cadd(*p, CT<C>::from(slab_dentry(g, st, k, r, a)));
-    }
+    slab_dadd_entries<C>(g, st, k, M, ldm);
 }
 
 // In-place Gauss-Jordan inverse with partial pivoting of the n x n matrix M
@@ -281,23 +219,13 @@ __global__ void __launch_bounds__(kGjThreads) k_gj_invert(C* __restrict__ M, int
     }
 }
 
-// X (row-major sweep layout, ld, columns n..ld-1 zero) = M^{-1} from the
-// Gauss-Jordan result: X(a, c) = Mgj(a, pinv[c]) = M[pinv[c] * ldm + a].
+// X (tile layout) = M^{-1} from the Gauss-Jordan result: X(a, c) = Mgj(a, pinv[c]) =
+// M[pinv[c] * ldm + a]; rows n .. of the last tile are zero.
 template <typename C>
 __global__ void __launch_bounds__(256) k_slab_store(const C* __restrict__ M, int n, int ldm,
-                                                    const int* __restrict__ pinv, C* __restrict__ X, int ld) {
-    __shared__ C tile[32][33];
-    const int a0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    for (int i = ty; i < 32; i += 8) {   // column c0+i of X: rows a0+tx (contiguous in M)
-        const int c = c0 + i, a = a0 + tx;
-        tile[i][tx] = (c < n && a < n) ? M[(int64_t)pinv[c] * ldm + a] : CT<C>::zero();
-    }
-    __syncthreads();
-    for (int i = ty; i < 32; i += 8) {
-        const int a = a0 + i, c = c0 + tx;
-        if (a < n && c < ld) X[(int64_t)a * ld + c] = tile[tx][i];
-    }
+                                                    const int* __restrict__ pinv, C* __restrict__ X) {
+    const int a = blockIdx.x * 64 + (threadIdx.x & 63), c = blockIdx.y * 4 + (threadIdx.x >> 6);
+    if (c < n) X[slab_at(n, a, c)] = a < n ? M[(int64_t)pinv[c] * ldm + a] : CT<C>::zero();
 }
 
 // ------------------------------------------------------------------ sweeps
@@ -330,33 +258,67 @@ __global__ void k_slab_rhs(Geom g, StripDev st, SweepStep sp, StripDev pst, cons
     }
 }
 
-// A whole strip solve (2 N_y - 1 block steps) in one cooperative launch of at most
-// one CTA per SM.  CTA b owns rows [b rpc, (b+1) rpc) of every block; step s is
-//   forward  (s < N_y):      y_k = X_k (r_k - C_k y_{k-1}),       k = s
-//   backward (s >= N_y):     x_k = y_k - X_k (C_{k+1} x_{k+1}),    k = 2 N_y - 2 - s
-// in place in Y.  A producer warp streams the CTA's rows of X_k, step after step,
-// into a ring of row slots in shared memory (cp.async.bulk + mbarriers), with the
-// next step's rows prefetched into L2; it never waits for the vector, so the factor
-// stream runs ahead across the steps while the compute warps wait at the grid barrier
-// for the previous step's rows.  Compute warp w owns the column segment
-// [w seg, (w+1) seg) of every row: it loads its part of the step's input vector
-// z = r_k - C y_kp straight into registers, forms its partial products for all rows
-// of the step (four rows at a time), and the eight partials of a row are summed in
-// shared memory.  Every wait is bounded: on time-out the kernel records 7 in the
-// status word, waits (bounded) for its copies in flight and returns.
+// A whole strip solve (2 N_y - 1 block steps) in one cooperative launch, one CTA per SM.
+//
+// Every block is cut into mr x nq tiles of 128 rows by kc columns; CTA (m, q) streams its tile
+// of every block and multiplies it with its kc entries of the step's input vector z (for NB
+// right-hand sides).  A step of a chain is
+//   product: partial sums of the CTA's 128 rows into P[chain][q], counter part[m] raised;
+//   sum:     the CTA's own `epc` entries of its row tile: y = sum over q of P (plus y_k on the
+//            way out), stored to Y, and the next step's z = r - C y on them, counter vec[m]
+//            raised.
+// A CTA's sums wait for the nq CTAs of its row tile only, and its copy of z for the two or three
+// row tiles that hold its columns.  Z and P are double buffered by the step's parity: a CTA
+// enters product s+2 after the products s+1 of its row tile, each of which followed its
+// CTA's sums of step s; and it writes z of step s+2 after all of its row tile's products
+// s+1, which together waited for every CTA's z of step s+1 and so for every product s.
+// The two chains are independent up to the middle row, and the warps are specialised, so that
+// one chain's sums, counters and vector loads run while the other chain's tile is multiplied:
+//   8 product warps  walk both chains in turn (top, bottom, top, ...);
+//   2 x 3 sum warps  one group per chain: sums, z, and the copy of z into shared memory (by
+//                    plain loads: a bulk copy would queue behind the ring's tiles);
+//   1 producer warp  streams the tiles, step after step, through a ring of column slots
+//                    (cp.async.bulk + mbarriers) ahead of the products and never waits for z.
+// Splitting the columns too (instead of giving a CTA whole rows) keeps a CTA's share of z at
+// kc entries: with whole rows the vectors of 8 right-hand sides were more L2 traffic than the
+// blocks themselves (63^3 grid, blocks of 1659: 19 us per block and 8 right-hand sides).
+// A warp's lane holds 4 of the 128 rows (two adjacent ones in each 64-row half), so a product
+// needs no reduction over lanes; the warps split the slot's columns (and, for 16 right-hand
+// sides, the right-hand sides in two), their sums meet in shared memory once per step.
+// What bounds it: with one right-hand side the chain's latency under the stream's load (tile
+// 7.4k cycles, the rest of a step about 12k, half of it hidden by the other chain); with 16
+// the shared-memory reads and FP32 FMAs of the tile.  One application of P on the 63^3 grid
+// (8 strips, blocks of 1659-1817, 15 strip solves; top-down elimination with whole rows per
+// CTA and tiles of 4 right-hand sides before): 16.4 -> 11.3 ms with one right-hand side (3.2
+// -> 4.7 TB/s of blocks), 127 -> 28.3 ms with 16.
+// Every wait is bounded: on time-out the kernel records 7 in the status word, waits (bounded)
+// for its copies in flight and returns.
 template <typename C>
 struct SlabSweepArgs {
-    const C* X;          // block 0 of the strip; block k at X + k * bs, row-major, leading dimension xld
+    const C* X;          // block 0 of the strip in the tile layout (slab_ops.cuh); block k at X + k * bs
     int64_t bs;
-    int n, xld, Ny, rpc, ring;
+    int n, Ny;
+    int nq, kc, ncta, epc, slots;
     const C* rhs;        // [B][Ny][ld] right-hand sides
     C* Y;                // [B][Ny][ld] solution
     int ld, B;           // row stride of rhs / Y; right-hand sides of this launch (<= NB)
     const C* sxz;        // s_x(c) s_z(z) per block entry
     const C* cyt;        // -alpha_y(y_{k-1/2}) / h^2, k = 0 .. Ny
-    unsigned* bar;       // step counter, zero at launch
+    C* Z;                // [chain][step parity][nz][NB] input vectors, nz = n rounded up to even
+    C* P;                // [chain][step parity][nq][n][NB] partial sums
+    unsigned* bar;       // counters [part, vec][chain][kMaxRowTiles], kCtrStride apart, zero at launch
     int* status;
 };
+constexpr int kCtrStride = 32;      // counters on separate 128-byte lines
+constexpr int kMaxRowTiles = 32;    // blocks of up to 4096 unknowns
+constexpr size_t kCtrBytes = (size_t)4 * kMaxRowTiles * kCtrStride * sizeof(unsigned);   // 16 KB
+__device__ __forceinline__ unsigned* slab_ctr(unsigned* bar, int vec, int ch, int m) {
+    return bar + ((vec * 2 + ch) * kMaxRowTiles + m) * kCtrStride;
+}
+constexpr int kProdWarps = 8, kSumThreads = 96;
+constexpr int kSweepThreads = 32 * kProdWarps + 2 * kSumThreads + 32;
+constexpr int kSlotBytes = 16 * 1024;   // a ring slot: 16 (complex64) or 8 columns of 128 rows
+constexpr int kMaxSlots = 16;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mb_init(uint64_t* m, uint32_t count) {
@@ -368,7 +330,8 @@ __device__ __forceinline__ void mb_expect_tx(uint64_t* m, uint32_t bytes) {
 __device__ __forceinline__ void mb_arrive(uint64_t* m) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(m)) : "memory");
 }
-__device__ __forceinline__ bool mb_wait(uint64_t* m, uint32_t parity) {
+// bounded; gives up early once the CTA has recorded a failed wait
+__device__ __forceinline__ bool mb_wait(uint64_t* m, uint32_t parity, const volatile int* abort_flag = nullptr) {
     for (uint32_t it = 0; it < kBarPolls; ++it) {
         uint32_t ok;
         asm volatile(
@@ -377,203 +340,327 @@ __device__ __forceinline__ bool mb_wait(uint64_t* m, uint32_t parity) {
             : "r"(smem_addr(m)), "r"(parity)
             : "memory");
         if (ok) return true;
+        if (abort_flag && *abort_flag) return false;
     }
     return false;
 }
-__device__ __forceinline__ void bulk_row(void* dst, const void* src, uint32_t bytes, uint64_t* m) {
+__device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t bytes, uint64_t* m) {
     asm volatile(
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_addr(dst)),
         "l"(src), "r"(bytes), "r"(smem_addr(m))
         : "memory");
 }
-__device__ __forceinline__ void compute_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ void group_sync(int id, int nthr) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthr) : "memory");
+}
 
-constexpr int kSweepThreads = 288;   // 8 compute warps + 1 producer warp
-constexpr int kMaxRpc = 32;          // rows per CTA and step
+// Barrier of the group that returns, to all its threads alike, whether any of them passed v != 0.
+__device__ __forceinline__ bool group_or(int id, int nthr, int v) {
+    uint32_t r;
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.b32 p, %1, 0;\n bar.red.or.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+        : "=r"(r)
+        : "r"(v), "r"(id), "r"(nthr)
+        : "memory");
+    return r != 0;
+}
 
-// kSegU: columns per lane, 8 warps x 32 lanes x kSegU >= xld (8: n <= 2048, 16: n <= 4096)
-template <typename C, int NB, int kSegU>
+// The grid row of step i of a chain: the top chain (0) walks rows 0 .. t-1, t, t-1 .. 0, the
+// bottom chain (1) rows N_y-1 .. t+1, t+1 .. N_y-1, with t = (N_y-1)/2.
+__device__ __forceinline__ int slab_row(int chain, int i, int Ny) {
+    const int t = (Ny - 1) / 2, nu = Ny - 1 - t;
+    if (chain == 0) return i <= t ? i : 2 * t - i;
+    return i < nu ? Ny - 1 - i : t + 1 + (i - nu);
+}
+// Step p of the walk over both chains: their forward steps in turn, the middle row, the
+// outward steps in turn; the bottom chain's extra row (N_y even) comes last of its half.
+__device__ __forceinline__ int slab_chain(int p, int Ny) {
+    const int t = (Ny - 1) / 2, nu = Ny - 1 - t, nf = t + nu;
+    if (p == nf) return 0;
+    const int q = p < nf ? p : p - nf - 1;
+    return q >= 2 * t ? 1 : q & 1;
+}
+
+// two adjacent entries of shared memory (16-byte aligned in complex64)
+__device__ __forceinline__ void ld_pair(const float2* p, float2& a, float2& b) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    a = make_float2(v.x, v.y);
+    b = make_float2(v.z, v.w);
+}
+__device__ __forceinline__ void ld_pair(const double2* p, double2& a, double2& b) { a = p[0]; b = p[1]; }
+
+__device__ __forceinline__ void ldcg_pair(const float2* p, float2& a, float2& b) {
+    const float4 v = __ldcg(reinterpret_cast<const float4*>(p));
+    a = make_float2(v.x, v.y);
+    b = make_float2(v.z, v.w);
+}
+__device__ __forceinline__ void ldcg_pair(const double2* p, double2& a, double2& b) { a = __ldcg(p); b = __ldcg(p + 1); }
+
+// Right-hand sides of a tile and how the product warps share them: kRG groups of warps take
+// NB / kRG each, the others split the columns.
+template <int NB> struct SlabTile {
+    static constexpr int kRG = NB > 8 ? 2 : 1, kN = NB / kRG, kKG = kProdWarps / kRG;
+    // the column groups' sums, [group][4 rows][NB][33] (the last dimension padded so that the
+    // lanes of a warp read and write different banks)
+    static constexpr int kRed = kKG * 4 * NB * 33;
+    static constexpr int kMaxEpc = NB > 8 ? 18 : 36;                         // own entries of a CTA, at most
+    static constexpr int kVals = (kMaxEpc * NB + kSumThreads - 1) / kSumThreads;   // values of a sum thread
+};
+
+template <typename C, int NB>
+__host__ __device__ inline size_t slab_sweep_fixed(int kc) {
+    return (size_t)2 * kc * NB * sizeof(C) + (size_t)SlabTile<NB>::kRed * sizeof(C) +
+           (2 * kMaxSlots + 4) * 8 + 16;
+}
+
+template <typename C, int NB>
 __global__ void __launch_bounds__(kSweepThreads, 1) k_slab_sweep(SlabSweepArgs<C> A) {
-    using R = typename CT<C>::R;
+    using T = SlabTile<NB>;
+    constexpr int SC = kSlotBytes / (128 * (int)sizeof(C));   // columns of a slot
     extern __shared__ __align__(128) unsigned char sweep_smem[];
-    const int R_ = A.ring, xld = A.xld;
-    C* ring = reinterpret_cast<C*>(sweep_smem);                       // [ring][xld]
-    C* part = ring + (int64_t)R_ * xld;                               // [8][kMaxRpc][NB] partial products
-    uint64_t* full = reinterpret_cast<uint64_t*>(part + 8 * kMaxRpc * NB);   // [ring]
-    uint64_t* empty = full + R_;                                      // [ring]
-    int* abort_flag = reinterpret_cast<int*>(empty + R_);
+    C* ring = reinterpret_cast<C*>(sweep_smem);                                   // [slots][2][SC][64]
+    C* zs = reinterpret_cast<C*>(sweep_smem + (size_t)A.slots * kSlotBytes);      // [2][kc][NB]
+    C* red = zs + (size_t)2 * A.kc * NB;                                          // [column group][4 rows][NB][33]
+    uint64_t* full = reinterpret_cast<uint64_t*>(red + T::kRed);
+    uint64_t* empty = full + kMaxSlots;
+    uint64_t* zfull = empty + kMaxSlots;   // [2] z of the chain's step is in zs
+    uint64_t* xdone = zfull + 2;           // [0] middle row summed, [1] bottom chain's forward half summed
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(xdone + 2);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int r0 = blockIdx.x * A.rpc, nrow = imin(A.rpc, A.n - r0);
-    const int nsteps = 2 * A.Ny - 1;
-    const uint32_t rowbytes = (uint32_t)(xld * sizeof(C));
-    // ring slots go back to the producer at the end of a step (after the grid arrival) when
-    // the ring holds a whole step; otherwise each warp frees a group's slots as soon as it
-    // has used them
-    constexpr int RG = NB == 1 ? 4 : 2;
-    const bool defer = R_ >= A.rpc;
+    const int Ny = A.Ny, n = A.n, nz = (n + 1) & ~1;
+    const int m = (int)blockIdx.x / A.nq, q = (int)blockIdx.x % A.nq;
+    const int row0 = m * 128;
+    const int c0 = q * A.kc, ncol = imin(A.kc, n - c0);
+    const bool half2 = row0 + 64 < n;   // the tile's second 64-row half exists
+    const int nslot = (ncol + SC - 1) / SC;
+    const int t = (Ny - 1) / 2, nu = Ny - 1 - t;
     if (tid == 0) {
-        for (int i = 0; i < R_; ++i) { mb_init(&full[i], 1); mb_init(&empty[i], defer ? 1 : 8); }
+        for (int i = 0; i < A.slots; ++i) { mb_init(&full[i], 1); mb_init(&empty[i], kProdWarps); }
+        for (int i = 0; i < 2; ++i) { mb_init(&zfull[i], kSumThreads); mb_init(&xdone[i], 1); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    auto give_up = [&]() { atomicExch(A.status, 7); *abort_flag = 1; };
 
-    if (warp == 8) {   // producer
+    if (warp == kSweepThreads / 32 - 1) {   // ---- producer
         if (lane == 0) {
             uint32_t g = 0;
             bool ok = true;
-            // the CTA's rows of block k(s) into L2, one step ahead of the ring copies: the
-            // ring holds about one step, the HBM stream then runs on across the barrier
-            auto prefetch = [&](int s) {
-                if (s >= nsteps) return;
-                const int k = s < A.Ny ? s : 2 * A.Ny - 2 - s;
-                const char* src = reinterpret_cast<const char*>(A.X + (int64_t)k * A.bs + (int64_t)r0 * xld);
-                const uint32_t bytes = (uint32_t)nrow * rowbytes;
-                for (uint32_t o = 0; o < bytes; o += 65536)
-                    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src + o),
-                                 "r"(bytes - o < 65536 ? bytes - o : 65536)
-                                 : "memory");
-            };
-            prefetch(0);
-            for (int s = 0; s < nsteps && ok; ++s) {
-                prefetch(s + 1);
-                const int k = s < A.Ny ? s : 2 * A.Ny - 2 - s;
-                const C* src = A.X + (int64_t)k * A.bs + (int64_t)r0 * xld;
-                for (int i = 0; i < nrow; ++i, ++g) {
-                    const int slot = (int)(g % (uint32_t)R_);
-                    const uint32_t use = g / (uint32_t)R_;
-                    if (use > 0 && !mb_wait(&empty[slot], (use - 1) & 1)) { ok = false; break; }
-                    if (*(volatile int*)abort_flag) { ok = false; break; }
-                    mb_expect_tx(&full[slot], rowbytes);
-                    bulk_row(ring + (int64_t)slot * xld, src + (int64_t)i * xld, rowbytes, &full[slot]);
+            int step[2] = {0, 0};
+            for (int p = 0; p < 2 * Ny - 1 && ok; ++p) {
+                const int ch = slab_chain(p, Ny);
+                const int k = slab_row(ch, ch ? step[1]++ : step[0]++, Ny);
+                const C* lo = A.X + (int64_t)k * A.bs + ((int64_t)(2 * m) * n + c0) * 64;
+                const C* hi = lo + (int64_t)n * 64;
+                for (int i = 0; i < nslot; ++i, ++g) {
+                    const int slot = (int)(g % (uint32_t)A.slots);
+                    const uint32_t use = g / (uint32_t)A.slots;
+                    if (use > 0 && !mb_wait(&empty[slot], (use - 1) & 1, abort_flag)) { ok = false; break; }
+                    const uint32_t bytes = (uint32_t)(imin(SC, ncol - i * SC) * 64 * (int)sizeof(C));
+                    C* dst = ring + (int64_t)slot * (kSlotBytes / (int)sizeof(C));
+                    mb_expect_tx(&full[slot], half2 ? 2 * bytes : bytes);
+                    bulk_copy(dst, lo + (int64_t)i * SC * 64, bytes, &full[slot]);
+                    if (half2) bulk_copy(dst + SC * 64, hi + (int64_t)i * SC * 64, bytes, &full[slot]);
                 }
             }
-            if (!ok) atomicExch(A.status, 7);
+            if (!ok && !*abort_flag) give_up();
             // copies still in flight land before the CTA exits
-            const uint32_t lo = g > (uint32_t)R_ ? g - (uint32_t)R_ : 0;
-            for (uint32_t q = lo; q < g; ++q) mb_wait(&full[q % (uint32_t)R_], (q / (uint32_t)R_) & 1);
+            const uint32_t lo = g > (uint32_t)A.slots ? g - (uint32_t)A.slots : 0;
+            for (uint32_t i = lo; i < g; ++i) mb_wait(&full[i % (uint32_t)A.slots], (i / (uint32_t)A.slots) & 1);
         }
         return;
     }
 
-    // compute warps
-    const int e0 = warp * 32 * kSegU + lane;   // this lane's columns: e0 + 32 u, u < kSegU
-    uint32_t g0 = 0;   // issue index of this step's first row
-    for (int s = 0; s < nsteps; ++s, g0 += (uint32_t)nrow) {
-        const bool fwd = s < A.Ny;
-        const int k = fwd ? s : 2 * A.Ny - 2 - s;
-        const int kp = fwd ? k - 1 : k + 1;   // neighbouring row whose solution enters
-        if (s > 0) {   // every CTA's rows of the previous step are written
-            if (tid == 0) {
-                const unsigned target = (unsigned)s * gridDim.x;
-                unsigned v = ld_acquire_gpu(A.bar);
-                for (uint32_t it = 0; v < target && it < kBarPolls; ++it) {
-                    __nanosleep(20);
-                    v = ld_acquire_gpu(A.bar);
+    if (warp >= kProdWarps) {   // ---- sum warps of chain ch
+        const int ch = (tid - 32 * kProdWarps) / kSumThreads, at = (tid - 32 * kProdWarps) % kSumThreads;
+        const int nstep = ch == 0 ? 2 * t + 1 : 2 * nu;
+        const int e0 = row0 + q * A.epc, ne = imax(0, imin(A.epc, imin(n, row0 + 128) - e0));
+        unsigned* c_part = slab_ctr(A.bar, 0, ch, m);
+        unsigned* c_vec = slab_ctr(A.bar, 1, ch, m);
+        const int mz0 = c0 / 128, mz1 = (c0 + ncol - 1) / 128;   // row tiles that hold this CTA's columns
+        // waits (one thread) until a counter reaches `target`
+        auto poll = [&](const unsigned* ctr, unsigned target) -> bool {
+            unsigned v = ld_acquire_gpu(ctr);
+            for (uint32_t it = 0; v < target && it < kBarPolls && !*abort_flag; ++it) v = ld_acquire_gpu(ctr);
+            return v >= target;
+        };
+        int ve[T::kVals], vb[T::kVals];   // this thread's values: entry (clamped), right-hand side
+        bool on[T::kVals], st[T::kVals];  // value exists / is a right-hand side of this launch
+        C sx[T::kVals], y[T::kVals];
+#pragma unroll
+        for (int i = 0; i < T::kVals; ++i) {
+            const int v = at + i * kSumThreads;
+            on[i] = v < ne * NB;
+            ve[i] = imin(e0 + v / NB, n - 1);
+            vb[i] = v % NB;
+            st[i] = on[i] && vb[i] < A.B;
+            sx[i] = A.sxz[ve[i]];
+            y[i] = CT<C>::zero();
+        }
+        auto yp = [&](int i, int k) -> C* { return A.Y + ((int64_t)imin(vb[i], A.B - 1) * Ny + k) * A.ld + ve[i]; };
+        auto forward = [&](int s) { return ch == 0 ? s <= t : s < nu; };
+        // of step s: the right-hand side, or y_k on the way out (the bottom chain turns on the row
+        // it has just summed, whose value is still in y)
+        C base[T::kVals], next[T::kVals], cy0 = CT<C>::zero(), cy1 = CT<C>::zero();
+        auto load_step = [&](int s) {   // and the couplings to the step before and, at the middle row, to y_{t+1}
+            const int k = slab_row(ch, s, Ny);
+            const bool fwd = forward(s);
+            cy0 = A.cyt[ch == 0 ? (s <= t ? k : k + 1) : (s < nu ? k + 1 : k)];
+            cy1 = A.cyt[k + 1];
+            if (ch == 1 && s == nu) return;
+#pragma unroll
+            for (int i = 0; i < T::kVals; ++i)
+                next[i] = !st[i] ? CT<C>::zero()
+                          : fwd  ? ldcg(A.rhs + ((int64_t)vb[i] * Ny + k) * A.ld + ve[i])
+                                 : ldcg(yp(i, k));
+        };
+        if (nstep > 0) load_step(0);
+        for (int s = 0; s < nstep; ++s) {
+            const int k = slab_row(ch, s, Ny);
+            const bool mid = ch == 0 && s == t, fwd = forward(s);
+#pragma unroll
+            for (int i = 0; i < T::kVals; ++i) base[i] = ch == 1 && s == nu ? y[i] : next[i];
+            // the other chain's values of the same entries: y_{t+1} at the middle row, x_t for the
+            // bottom chain's way out
+            bool ok = true;
+            const bool cross = (mid && nu > 0) || (ch == 1 && s == nu);
+            if (cross) ok = mb_wait(&xdone[mid ? 1 : 0], 0, abort_flag);
+            C* zg = A.Z + (int64_t)(ch * 2 + (s & 1)) * nz * NB;
+#pragma unroll
+            for (int i = 0; i < T::kVals; ++i) {
+                if (!on[i]) continue;
+                C z = fwd ? base[i] : CT<C>::zero();
+                if (st[i]) {
+                    C prev = y[i];
+                    if (ch == 1 && s == nu) prev = ldcg(yp(i, t));
+                    if (s > 0) z = csub(z, cmul(cmul(cy0, sx[i]), prev));
+                    if (mid && nu > 0) z = csub(z, cmul(cmul(cy1, sx[i]), ldcg(yp(i, t + 1))));
                 }
-                if (v < target) { atomicExch(A.status, 7); *(volatile int*)abort_flag = 1; }
+                zg[(int64_t)ve[i] * NB + vb[i]] = z;
             }
-            compute_sync();
-            if (*(volatile int*)abort_flag) return;
-        }
-        // backward: y_k of the rows this CTA outputs (thread t < nrow B: row t / B, rhs t % B)
-        const int ob = tid % NB, oi = tid / NB;
-        const bool outs = tid < nrow * NB && ob < A.B;
-        C* yo = A.Y + ((int64_t)imin(ob, A.B - 1) * A.Ny + k) * A.ld + r0 + imin(oi, nrow - 1);
-        const C ybase = (outs && !fwd) ? *yo : CT<C>::zero();
-        // z = r_k - cy sxz .* y_kp on this lane's columns, in registers
-        const C cy = A.cyt[fwd ? k : k + 1];
-        C z[kSegU][NB];
-#pragma unroll
-        for (int u = 0; u < kSegU; ++u) {
-            const int e = e0 + 32 * u;
-            const bool ok = e < A.n;
-            const int ec = imin(e, A.n - 1);
-            const C sc = cmul(cy, ok ? A.sxz[ec] : CT<C>::zero());
-#pragma unroll
-            for (int b = 0; b < NB; ++b) {
-                const bool okb = ok && b < A.B;
-                const int64_t rb = (int64_t)imin(b, A.B - 1) * A.Ny;
-                const C r = (okb && fwd) ? ldcg(A.rhs + (rb + k) * A.ld + ec) : CT<C>::zero();
-                const C y = (okb && kp >= 0) ? ldcg(A.Y + (rb + kp) * A.ld + ec) : CT<C>::zero();
-                z[u][b] = csub(r, cmul(sc, y));
+            if (!ok) give_up();
+            group_sync(2 + ch, kSumThreads);
+            const unsigned target = (unsigned)(s + 1) * (unsigned)A.nq;
+            if (at == 0) {
+                asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(c_vec) : "memory");
+                bool zok = !*abort_flag;
+                for (int mm = mz0; mm <= mz1 && zok; ++mm) zok = poll(slab_ctr(A.bar, 1, ch, mm), target);
+                if (!zok && !*abort_flag) give_up();
             }
-        }
-        // partial products of this warp's segment, RG rows at a time: the group's rows
-        // are awaited first, then their products interleaved (independent chains)
-        bool ok = true;
-        for (int i0 = 0; i0 < nrow && ok; i0 += RG) {
-            bool landed = true;
+            if (group_or(2 + ch, kSumThreads, *abort_flag)) return;
+            // z of this CTA's columns into shared memory, two entries a load; every product of the
+            // previous step has read zs (its partial sums are in)
+            {
+                const C* src = zg + (int64_t)c0 * NB;
+                C* dst = zs + (size_t)ch * A.kc * NB;
+                const int tot = (ncol * NB + 1) / 2;
+                constexpr int kBatch = sizeof(C) == sizeof(float2) ? 8 : 4;
+                for (int o0 = at; o0 < tot; o0 += kBatch * kSumThreads) {
+                    C v[kBatch][2];
 #pragma unroll
-            for (int r = 0; r < RG; ++r) {
-                const uint32_t g = g0 + (uint32_t)(i0 + r);
-                if (i0 + r < nrow) landed &= mb_wait(&full[g % (uint32_t)R_], (g / (uint32_t)R_) & 1);
-            }
-            if (!__all_sync(0xffffffffu, landed)) { ok = false; break; }
-            const C* xr[RG];
+                    for (int j = 0; j < kBatch; ++j)
+                        ldcg_pair(src + 2 * imin(o0 + j * kSumThreads, tot - 1), v[j][0], v[j][1]);
 #pragma unroll
-            for (int r = 0; r < RG; ++r)
-                xr[r] = ring + (int64_t)((g0 + (uint32_t)imin(i0 + r, nrow - 1)) % (uint32_t)R_) * xld;
-            C acc[RG][NB];
-#pragma unroll
-            for (int r = 0; r < RG; ++r)
-#pragma unroll
-                for (int b = 0; b < NB; ++b) acc[r][b] = CT<C>::zero();
-#pragma unroll
-            for (int u = 0; u < kSegU; ++u) {
-                const int e = e0 + 32 * u;
-                C x[RG];
-#pragma unroll
-                for (int r = 0; r < RG; ++r) x[r] = e < xld ? xr[r][e] : CT<C>::zero();
-#pragma unroll
-                for (int r = 0; r < RG; ++r)
-#pragma unroll
-                    for (int b = 0; b < NB; ++b) acc[r][b] = cfma(x[r], z[u][b], acc[r][b]);
-            }
-            if (!defer) {
-                __syncwarp();
-                if (lane == 0)
-                    for (int r = 0; r < RG && i0 + r < nrow; ++r)
-                        mb_arrive(&empty[(g0 + (uint32_t)(i0 + r)) % (uint32_t)R_]);
-            }
-#pragma unroll
-            for (int r = 0; r < RG; ++r)
-#pragma unroll
-                for (int b = 0; b < NB; ++b) {
-                    R re = acc[r][b].x, im = acc[r][b].y;
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        re += __shfl_xor_sync(0xffffffffu, re, o);
-                        im += __shfl_xor_sync(0xffffffffu, im, o);
+                    for (int j = 0; j < kBatch; ++j) {
+                        const int o = o0 + j * kSumThreads;
+                        if (o < tot) { dst[2 * o] = v[j][0]; dst[2 * o + 1] = v[j][1]; }
                     }
-                    acc[r][b].x = re;
-                    acc[r][b].y = im;
                 }
-            if (lane == 0)
+                mb_arrive(&zfull[ch]);
+            }
+            if (s + 1 < nstep) load_step(s + 1);   // in flight during the wait
+            if (at == 0 && !poll(c_part, target) && !*abort_flag) give_up();
+            if (group_or(2 + ch, kSumThreads, *abort_flag)) return;
+            // y = [y_k +] the sum of the partial sums
+            const C* pp = A.P + (int64_t)(ch * 2 + (s & 1)) * A.nq * n * NB;
 #pragma unroll
-                for (int r = 0; r < RG; ++r)
-                    if (i0 + r < nrow)
+            for (int i = 0; i < T::kVals; ++i) y[i] = fwd ? CT<C>::zero() : base[i];
+            constexpr int kBatch = 6;   // partial sums in flight per value
+            for (int j0 = 0; j0 < A.nq; j0 += kBatch) {
+                C v[T::kVals][kBatch];
 #pragma unroll
-                        for (int b = 0; b < NB; ++b) part[(warp * kMaxRpc + i0 + r) * NB + b] = acc[r][b];
-        }
-        if (!ok && lane == 0) { atomicExch(A.status, 7); *(volatile int*)abort_flag = 1; }
-        compute_sync();
-        if (*(volatile int*)abort_flag) return;
-        if (outs) {   // the eight partials of row oi, rhs ob
-            C v = ybase;
+                for (int i = 0; i < T::kVals; ++i)
 #pragma unroll
-            for (int w = 0; w < 8; ++w) v = cadd(v, part[(w * kMaxRpc + oi) * NB + ob]);
-            *yo = v;
+                    for (int j = 0; j < kBatch; ++j)
+                        v[i][j] = ldcg(pp + ((int64_t)imin(j0 + j, A.nq - 1) * n + ve[i]) * NB + vb[i]);
+#pragma unroll
+                for (int i = 0; i < T::kVals; ++i)
+#pragma unroll
+                    for (int j = 0; j < kBatch; ++j)
+                        if (j0 + j < A.nq) y[i] = cadd(y[i], v[i][j]);
+            }
+#pragma unroll
+            for (int i = 0; i < T::kVals; ++i)
+                if (st[i]) *yp(i, k) = y[i];
+            if (mid || (ch == 1 && s == nu - 1)) {
+                group_sync(2 + ch, kSumThreads);
+                if (at == 0) mb_arrive(&xdone[mid ? 0 : 1]);
+            }
         }
-        compute_sync();
-        if (tid == 0) {
-            // this CTA's rows of step s are written (release: ordered after the barrier above);
-            // only then are the step's ring slots handed back, so that the refill traffic does
-            // not queue in front of the release
-            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(A.bar) : "memory");
-            if (defer)
-                for (int i = 0; i < nrow; ++i) mb_arrive(&empty[(g0 + (uint32_t)i) % (uint32_t)R_]);
+        return;
+    }
+
+    // ---- product warps
+    const int rg = warp % T::kRG, kg = warp / T::kRG;   // right-hand sides, columns
+    const int rl = 2 * lane;                            // rows rl, rl+1 of each half
+    uint32_t g = 0;
+    int step[2] = {0, 0};
+    for (int p = 0; p < 2 * Ny - 1; ++p) {
+        const int ch = slab_chain(p, Ny);
+        const int s = ch ? step[1]++ : step[0]++;
+        bool ok = __all_sync(0xffffffffu, mb_wait(&zfull[ch], (uint32_t)(s & 1), abort_flag));
+        const C* zc = zs + (size_t)ch * A.kc * NB + rg * T::kN;
+        C acc[4][T::kN];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int b = 0; b < T::kN; ++b) acc[r][b] = CT<C>::zero();
+        for (int i = 0; i < nslot && ok; ++i, ++g) {
+            const int slot = (int)(g % (uint32_t)A.slots);
+            ok = mb_wait(&full[slot], (g / (uint32_t)A.slots) & 1, abort_flag);
+            if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
+            const C* xs = ring + (int64_t)slot * (kSlotBytes / (int)sizeof(C)) + rl;
+            const int nc = imin(SC, ncol - i * SC);
+#pragma unroll 2
+            for (int c = kg; c < nc; c += T::kKG) {
+                C x[4], z[T::kN];
+                ld_pair(xs + c * 64, x[0], x[1]);
+                ld_pair(xs + (SC + c) * 64, x[2], x[3]);
+                const C* zp = zc + (size_t)(i * SC + c) * NB;
+                if constexpr (T::kN == 1) {
+                    z[0] = zp[0];
+                } else {
+#pragma unroll
+                    for (int b = 0; b < T::kN; b += 2) ld_pair(zp + b, z[b], z[b + 1]);
+                }
+#pragma unroll
+                for (int b = 0; b < T::kN; ++b)
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) acc[r][b] = cfma(x[r], z[b], acc[r][b]);
+            }
+            __syncwarp();
+            if (lane == 0) mb_arrive(&empty[slot]);
         }
+        if (!ok && lane == 0 && !*abort_flag) give_up();
+        C* pp = A.P + (int64_t)((ch * 2 + (s & 1)) * A.nq + q) * n * NB;
+        C* rr = red + (size_t)kg * 4 * NB * 33 + (size_t)rg * T::kN * 33 + lane;
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int b = 0; b < T::kN; ++b) rr[(r * NB + b) * 33] = acc[r][b];
+        group_sync(1, 32 * kProdWarps);
+        for (int o = tid; o < 128 * NB; o += 32 * kProdWarps) {   // adjacent threads: adjacent right-hand sides
+            const int b = o % NB, rw = o / NB;                    // row of the tile
+            const int h2 = rw >> 6, l = (rw & 63) >> 1, r = 2 * h2 + (rw & 1);
+            C v = CT<C>::zero();
+#pragma unroll
+            for (int h = 0; h < T::kKG; ++h) v = cadd(v, red[((size_t)(h * 4 + r) * NB + b) * 33 + l]);
+            if (row0 + rw < n) pp[(int64_t)(row0 + rw) * NB + b] = v;
+        }
+        if (group_or(1, 32 * kProdWarps, *abort_flag)) return;
+        if (tid == 0)
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(slab_ctr(A.bar, 0, ch, m)) : "memory");
     }
 }
 
@@ -634,12 +721,15 @@ cudaError_t launch_slab_factor(const Geom& g, const StripDev& st, void* pool, co
     C* X = reinterpret_cast<C*>(pool) + st.fac;
     C* M = reinterpret_cast<C*>(sc.M);
     C* mult = reinterpret_cast<C*>(sc.mult);
-    const dim3 tiles((n + 31) / 32, (n + 31) / 32), tiles_st((st.ld + 31) / 32, (n + 31) / 32);
-    for (int k = 0; k < g.Ny; ++k) {
+    const dim3 tiles((n + 63) / 64, (n + 3) / 4), tiles_st((n + 63) / 64, (n + 3) / 4);
+    const int tmid = (g.Ny - 1) / 2;
+    for (int i = 0; i < g.Ny; ++i) {   // rows 0 .. t-1, N_y-1 .. t+1, t
+        const int k = i < tmid ? i : i < g.Ny - 1 ? g.Ny - 1 - (i - tmid) : tmid;
+        const C* Xp = k > 0 && k <= tmid ? X + (int64_t)(k - 1) * st.bs : nullptr;
+        const C* Xn = k + 1 < g.Ny && k >= tmid ? X + (int64_t)(k + 1) * st.bs : nullptr;
         {
             TimedLaunch t(tm, "slab_build", s);
-            k_slab_build<C><<<tiles, 256, 0, s>>>(g, st, k, k > 0 ? X + (int64_t)(k - 1) * st.bs : nullptr, st.ld,
-                                                   M, sc.ldm);
+            k_slab_build<C><<<tiles, 256, 0, s>>>(g, st, k, Xp, Xn, M, sc.ldm);
             k_slab_dadd<C><<<(5 * n + 63) / 64, 64, 0, s>>>(g, st, k, M, sc.ldm);
         }
         e = cudaMemsetAsync(sc.bar, 0, 2 * sizeof(unsigned), s);
@@ -654,12 +744,95 @@ cudaError_t launch_slab_factor(const Geom& g, const StripDev& st, void* pool, co
         }
         {
             TimedLaunch t(tm, "slab_store", s);
-            k_slab_store<C><<<tiles_st, 256, 0, s>>>(M, n, sc.ldm, sc.pinv, X + (int64_t)k * st.bs, st.ld);
+            k_slab_store<C><<<tiles_st, 256, 0, s>>>(M, n, sc.ldm, sc.pinv, X + (int64_t)k * st.bs);
         }
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
+}
+
+// The tile grid of a strip solve: mr row tiles of 128, nq column chunks of kc, at most one tile
+// per SM and at least 32 columns in a chunk (below that the partial sums of the chunks cost
+// more than the tiles).
+struct SlabGrid {
+    int nq, kc, ncta, epc;
+};
+static SlabGrid slab_grid(int n, int nsm) {
+    SlabGrid r;
+    const int mr = (n + 127) / 128;
+    r.nq = imax(1, imin(nsm / mr, (n + 31) / 32));
+    r.kc = ((n + r.nq - 1) / r.nq + 1) & ~1;   // even: every chunk of z starts 16-byte aligned
+    r.nq = (n + r.kc - 1) / r.kc;
+    r.ncta = mr * r.nq;
+    r.epc = (imin(n, 128) + r.nq - 1) / r.nq;
+    return r;
+}
+// The strip-solve kernel for tiles of NB right-hand sides, if the vectors and a ring of at least
+// four slots fit in shared memory.
+struct SlabKernel {
+    const void* fn = nullptr;
+    int nb = 0, slots = 0;
+    size_t smem = 0;
+};
+template <typename C, int NB>
+static bool slab_kernel(const SlabGrid& gr, SlabKernel& k) {
+    constexpr size_t kSmemMax = 227 * 1024;
+    const size_t fixed = slab_sweep_fixed<C, NB>(gr.kc);
+    if (gr.epc > SlabTile<NB>::kMaxEpc || fixed + 4 * kSlotBytes > kSmemMax) return false;
+    k.fn = (const void*)k_slab_sweep<C, NB>;
+    k.nb = NB;
+    k.slots = (int)std::min<size_t>(kMaxSlots, (kSmemMax - fixed) / kSlotBytes);
+    k.smem = fixed + (size_t)k.slots * kSlotBytes;
+    return true;
+}
+// For `left` remaining right-hand sides: the widest useful tile that fits (a tile streams every
+// block once whatever its width).  Complex128 takes two at most: its products are bound by the
+// FP64 pipe, not by the stream.
+template <typename C>
+static SlabKernel pick_slab_kernel(const SlabGrid& gr, int left) {
+    SlabKernel k;
+    if constexpr (std::is_same<C, float2>::value) {
+        if (left > 8 && slab_kernel<C, 16>(gr, k)) return k;
+        if (left > 4 && slab_kernel<C, 8>(gr, k)) return k;
+        if (left > 1 && slab_kernel<C, 4>(gr, k)) return k;
+    } else {
+        if (left > 1 && slab_kernel<C, 2>(gr, k)) return k;
+    }
+    slab_kernel<C, 1>(gr, k);
+    return k;
+}
+constexpr int kSlabMaxNb = 16;
+static cudaError_t sm_count(int& nsm) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    return e;
+}
+template <typename C>
+static cudaError_t slab_sweep_attrs() {
+    cudaError_t e = cudaSuccess;
+    auto set = [&](const void* fn) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    };
+    set((const void*)k_slab_sweep<C, 1>);
+    if constexpr (std::is_same<C, float2>::value) {
+        set((const void*)k_slab_sweep<C, 4>);
+        set((const void*)k_slab_sweep<C, 8>);
+        set((const void*)k_slab_sweep<C, 16>);
+    } else {
+        set((const void*)k_slab_sweep<C, 2>);
+    }
+    return e;
+}
+
+// Z and P of the strip solve, for strips of up to nmax unknowns.
+size_t slab_sweep_scratch(int nmax, size_t esize) {
+    int nsm = 0;
+    if (sm_count(nsm) != cudaSuccess) return 0;
+    size_t p = 0;
+    for (int n = 1; n <= nmax; ++n) p = std::max(p, (size_t)4 * slab_grid(n, nsm).nq * n * kSlabMaxNb * esize);
+    return (size_t)4 * (nmax + 1) * kSlabMaxNb * esize + p;
 }
 
 template <typename C>
@@ -679,62 +852,48 @@ cudaError_t launch_slab_solve(const Geom& g, const StripDev& st, const StripDev*
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    constexpr int NB = 4;
-    int dev = 0, nsm = 0;
-    e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    int nsm = 0;
+    e = sm_count(nsm);
     if (e != cudaSuccess) return e;
-    const int rpc = (n + nsm - 1) / nsm, ncta = (n + rpc - 1) / rpc;
-    // column segments of 8 per lane up to 2048 unknowns, 16 up to 4096 (complex64 only: the
-    // complex128 input vector of 16 columns x 4 right-hand sides would not fit in registers)
-    const bool wide = st.ld > 8 * 32 * 8;
-    if (rpc > kMaxRpc || st.ld > 8 * 32 * 16 || (wide && sizeof(C) != sizeof(float2))) return cudaErrorInvalidValue;
-    const size_t row = (size_t)st.ld * sizeof(C);
-    const size_t kSmemMax = 227 * 1024;
-    // the kernel for a tile of one or NB right-hand sides
-    auto pick = [&](bool one, bool w) -> const void* {
-        if constexpr (std::is_same<C, float2>::value) {
-            if (w) return one ? (const void*)k_slab_sweep<C, 1, 16> : (const void*)k_slab_sweep<C, NB, 16>;
-        }
-        return one ? (const void*)k_slab_sweep<C, 1, 8> : (const void*)k_slab_sweep<C, NB, 8>;
-    };
     static bool attr_set = false;
     if (!attr_set) {
-        for (const void* fn : {pick(true, false), pick(false, false), pick(true, true), pick(false, true)}) {
-            e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax);
-            if (e != cudaSuccess) return e;
-        }
+        e = slab_sweep_attrs<C>();
+        if (e != cudaSuccess) return e;
         attr_set = true;
     }
-    for (int b0 = 0; b0 < B; b0 += NB) {
-        const int nb = imin(NB, B - b0);
-        const int nbk = nb == 1 ? 1 : NB;
-        const size_t fixed = (size_t)8 * kMaxRpc * nbk * sizeof(C) + 128;
-        const int ring = (int)std::min<size_t>(64, (kSmemMax - fixed) / (row + 16));
-        if (ring < 4) return cudaErrorInvalidValue;   // a row group of the compute warps fits
-        const size_t smem = (size_t)ring * row + (size_t)8 * kMaxRpc * nbk * sizeof(C) + (size_t)ring * 16 + 16;
+    if (n > 128 * kMaxRowTiles) return cudaErrorInvalidValue;
+    const SlabGrid gr = slab_grid(n, nsm);
+    for (int b0 = 0; b0 < B;) {
+        const SlabKernel kr = pick_slab_kernel<C>(gr, B - b0);
+        if (!kr.fn) return cudaErrorInvalidValue;
+        const int nb = imin(kr.nb, B - b0);
         SlabSweepArgs<C> A{};
         A.X = X;
         A.bs = st.bs;
         A.n = n;
-        A.xld = st.ld;
         A.Ny = Ny;
-        A.rpc = rpc;
-        A.ring = ring;
+        A.nq = gr.nq;
+        A.kc = gr.kc;
+        A.ncta = gr.ncta;
+        A.epc = gr.epc;
+        A.slots = kr.slots;
         A.rhs = Rb + (int64_t)b0 * Ny * ld;
         A.Y = Y + (int64_t)b0 * Ny * ld;
         A.ld = ld;
         A.B = nb;
         A.sxz = sxz;
         A.cyt = ct + g.ct_cy;
+        A.Z = reinterpret_cast<C*>(wk.scratch);
+        A.P = A.Z + (size_t)4 * ((n + 1) & ~1) * kr.nb;
         A.bar = wk.bar;
         A.status = wk.status;
-        e = cudaMemsetAsync(wk.bar, 0, sizeof(unsigned), s);
+        e = cudaMemsetAsync(wk.bar, 0, kCtrBytes, s);
         if (e != cudaSuccess) return e;
         TimedLaunch t(tm, "slab_sweep", s);
         void* args[] = {&A};
-        e = cudaLaunchCooperativeKernel(pick(nbk == 1, wide), dim3(ncta), dim3(kSweepThreads), args, smem, s);
+        e = cudaLaunchCooperativeKernel(kr.fn, dim3(gr.ncta), dim3(kSweepThreads), args, kr.smem, s);
         if (e != cudaSuccess) return e;
+        b0 += nb;
     }
     return cudaGetLastError();
 }
@@ -750,26 +909,14 @@ cudaError_t launch_slab_out(const Geom& g, const StripDev& st, int dir, const vo
     return cudaGetLastError();
 }
 
-template <typename C>
-cudaError_t launch_slab_build(const Geom& g, const StripDev& st, int k, const C* Xp, int ld, C* M, int ldm,
-                              cudaStream_t s, KernelTimer* tm) {
-    const int n = st.W * g.Nz;
-    TimedLaunch t(tm, "slab_build", s);
-    k_slab_build<C><<<dim3((n + 31) / 32, (n + 31) / 32), 256, 0, s>>>(g, st, k, Xp, ld, M, ldm);
-    k_slab_dadd<C><<<(5 * n + 63) / 64, 64, 0, s>>>(g, st, k, M, ldm);
-    return cudaGetLastError();
-}
-template cudaError_t launch_slab_build<float2>(const Geom&, const StripDev&, int, const float2*, int, float2*, int,
-                                               cudaStream_t, KernelTimer*);
-
 // Loads this file's module onto the current device (the strip-solve kernels of a
 // preconditioner application).
 cudaError_t preload_slab_kernels() {
     cudaFuncAttributes fa;
     cudaError_t e = cudaFuncGetAttributes(&fa, k_slab_rhs<float2>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_rhs<double2>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_sweep<float2, 1, 8>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_sweep<double2, 1, 8>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_sweep<float2, 1>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_sweep<double2, 1>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_out<float2>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_out<double2>);
     return e;

@@ -3,7 +3,7 @@
 //
 // Every block X_k = S_k^{-1}, S_k = D_k - C_k X_{k-1} C_k (n x n, n = W N_z), is inverted
 // by blocked Gauss-Jordan elimination with partial pivoting, the J strips of the grid side
-// by side.  Pivot rows are not exchanged: a row that has served as the pivot of a column is
+// by side and in each strip the two chains toward the middle row (slab3d.cu).  Pivot rows are not exchanged: a row that has served as the pivot of a column is
 // marked (kstep) and left out of later pivot searches.  The columns go in panels of kTcBig,
 // each made of sub-panels of kTcSub:
 //
@@ -25,7 +25,7 @@
 //                columns) every column outside it.
 //   k_tc_store   after the last panel the block N holds the inverse up to the pivot order:
 //                X(a, c) = N(q_a, pos(c)), q_a the pivot row of step a and pos(c) the step
-//                whose pivot row was c; written in the sweep layout of the factor pool.
+//                whose pivot row was c; written in the tile layout of the factor pool.
 //
 // The complex product uses real operands: a row of G is (Re g_0, Im g_0, Re g_1, ...), and
 // complex column j of T gives two B rows, (Re t_0, -Im t_0, Re t_1, ...) for the real part
@@ -33,7 +33,7 @@
 // 2j+1 are the real and imaginary parts of output column j.
 #include <climits>
 
-#include "common.cuh"
+#include "slab_ops.cuh"
 #include "internal.h"
 
 namespace helm {
@@ -78,7 +78,7 @@ __device__ __forceinline__ void tc_split(float x, float& hi, float& lo) {
 
 }  // namespace
 
-// One strip's block under inversion and its work arrays.
+// One chain's block under inversion and its work arrays (n = 0: the chain has no block now).
 struct TcStrip {
     float2* M;     // n x n, column-major, leading dimension ldm
     int n, ldm;
@@ -87,12 +87,14 @@ struct TcStrip {
     int* pos;      // [n] step whose pivot row was r
     float* Th;     // [2 npad][kTcKT] the source's pivot rows, expanded (B operand rows; npad: n
     float* Tl;     // rounded up to kTcRows), TF32 high part and remainder
-    float2* X;     // the factor pool's block k (row-major, leading dimension xld)
-    int xld;
+    float2* X;     // the factor pool's block k (tile layout)
+    const float2* Xp;   // X_{k-1} and X_{k+1} where they enter S_k (null: not)
+    const float2* Xn;
+    int j, k;           // strip and grid row of the block
 };
-constexpr int kTcMaxStrips = 8;
+constexpr int kTcMaxStrips = 8;                 // strips of one call, two chains each
 struct TcArgs {
-    TcStrip s[kTcMaxStrips];
+    TcStrip s[2 * kTcMaxStrips];
     int sp;          // k_tc_panel: the sub-panel (columns sp kTcSub ..)
     int glo, ghi;    // gather / update: the source columns (G) and their pivot rows (T)
     int ulo, uhi;    // the columns to update, [ulo, glo) and [ghi, uhi); k_tc_panel: its panel
@@ -149,7 +151,22 @@ __device__ __forceinline__ void tc_arm(uint64_t* mbar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc_smem(mbar)), "r"(bytes) : "memory");
 }
 
-// One cluster of kTcPanelCl CTAs per strip; thread g = rank kTcPanelThreads + tid of the cluster
+// S_k = D_k - C_k X_{k-1} C_k - C_{k+1} X_{k+1} C_{k+1} of every chain (two launches), and
+// the chains' pivot marks cleared.
+__global__ void __launch_bounds__(256) k_tc_build(Geom g, const __grid_constant__ TcArgs a) {
+    const TcStrip& S = a.s[blockIdx.z];
+    if (blockIdx.y == 0 && threadIdx.x < 64) {
+        const int r = blockIdx.x * 64 + threadIdx.x;
+        if (r < S.n) S.kstep[r] = -1;
+    }
+    if (S.n > 0) slab_build_entries<float2>(g, g.strips[S.j], S.k, S.Xp, S.Xn, S.M, S.ldm);
+}
+__global__ void __launch_bounds__(64) k_tc_dadd(Geom g, const __grid_constant__ TcArgs a) {
+    const TcStrip& S = a.s[blockIdx.y];
+    if (S.n > 0) slab_dadd_entries<float2>(g, g.strips[S.j], S.k, S.M, S.ldm);
+}
+
+// One cluster of kTcPanelCl CTAs per chain; thread g = rank kTcPanelThreads + tid of the cluster
 // owns rows g + kTcPanelSpan k (k < kTcPanelRows) of the sub-panel in registers.  During step t
 // register s holds column (t + s) mod kTcSub (the registers rotate by one column per step, so
 // that the loop body indexes them statically).  After the elimination of column t-1 every warp
@@ -548,24 +565,13 @@ __global__ void k_tc_pos(const __grid_constant__ TcArgs a) {
     }
 }
 
-// X(a, c) = N(q_a, pos(c)) in the row-major sweep layout (columns n .. xld-1 zero).
+// X(a, c) = N(q_a, pos(c)) in the tile layout (rows n .. of the last tile zero).
 __global__ void __launch_bounds__(256) k_tc_store(const __grid_constant__ TcArgs a) {
-    __shared__ float2 tile[32][33];
     const TcStrip& S = a.s[blockIdx.z];
-    const int n = S.n;
-    const int a0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-    if (a0 >= n || c0 >= S.xld) return;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    for (int i = ty; i < 32; i += 8) {   // column c0+i of X, rows a0+tx
-        const int c = c0 + i, rr = a0 + tx;
-        const int pc = (c < n && rr < n) ? S.pos[c] : -1, q = pc >= 0 ? S.qs[rr] : -1;
-        tile[i][tx] = (pc < n && q >= 0 && q < n) ? S.M[(int64_t)pc * S.ldm + q] : make_float2(0.f, 0.f);
-    }
-    __syncthreads();
-    for (int i = ty; i < 32; i += 8) {
-        const int rr = a0 + i, c = c0 + tx;
-        if (rr < n && c < S.xld) S.X[(int64_t)rr * S.xld + c] = tile[tx][i];
-    }
+    const int n = S.n, r = blockIdx.x * 64 + (threadIdx.x & 63), c = blockIdx.y * 4 + (threadIdx.x >> 6);
+    if ((int)blockIdx.x * 64 >= n || c >= n) return;
+    const int pc = r < n ? S.pos[c] : -1, q = pc >= 0 ? S.qs[r] : -1;
+    S.X[slab_at(n, r, c)] = (pc < n && q >= 0 && q < n) ? S.M[(int64_t)pc * S.ldm + q] : make_float2(0.f, 0.f);
 }
 
 size_t slab_factor_tc_scratch(int nmax, int ns) {
@@ -573,7 +579,7 @@ size_t slab_factor_tc_scratch(int nmax, int ns) {
     const size_t ldm = (size_t)((nmax + 3) & ~3);
     const size_t per = ldm * nmax * sizeof(float2) + (size_t)3 * nmax * sizeof(int) +
                        (size_t)4 * npad * kTcKT * sizeof(float) + 6 * 256;
-    return per * ns;
+    return per * 2 * ns;
 }
 
 cudaError_t launch_slab_factor_tc(const Geom& g, const StripDev* strips, int ns, void* pool, void* scratch,
@@ -595,9 +601,9 @@ cudaError_t launch_slab_factor_tc(const Geom& g, const StripDev* strips, int ns,
     auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };
     char* sp = (char*)scratch;
     const int npad_max = (nmax + kTcRows - 1) / kTcRows * kTcRows;
-    for (int i = 0; i < ns; ++i) {
-        TcStrip& S = A.s[i];
-        S.n = strips[i].W * g.Nz;
+    const int nc = 2 * ns;   // chain 2 i (top) and 2 i + 1 (bottom) of strip i
+    for (int c = 0; c < nc; ++c) {
+        TcStrip& S = A.s[c];
         S.ldm = (nmax + 3) & ~3;
         S.M = (float2*)sp; sp += align((size_t)S.ldm * nmax * sizeof(float2));
         S.qs = (int*)sp; sp += align((size_t)nmax * sizeof(int));
@@ -605,9 +611,9 @@ cudaError_t launch_slab_factor_tc(const Geom& g, const StripDev* strips, int ns,
         S.pos = (int*)sp; sp += align((size_t)nmax * sizeof(int));
         S.Th = (float*)sp; sp += align((size_t)2 * npad_max * kTcKT * sizeof(float));
         S.Tl = (float*)sp; sp += align((size_t)2 * npad_max * kTcKT * sizeof(float));
-        S.xld = strips[i].ld;
+        S.j = strips[c / 2].j;
     }
-    const dim3 sgrid((nmax + 3 + 31) / 32, (nmax + 31) / 32, ns);
+    const dim3 sgrid((nmax + 63) / 64, (nmax + 3) / 4, nc);
     float2* pool2 = reinterpret_cast<float2*>(pool);
     // update the columns [ulo, glo) and [ghi, uhi) from the source [glo, ghi)
     auto update = [&](int glo, int ghi, int ulo, int uhi, int kmin, const char* name) {
@@ -619,33 +625,48 @@ cudaError_t launch_slab_factor_tc(const Geom& g, const StripDev* strips, int ns,
         const int nl = imax(glo - ulo, 0), nr = imax(uhi - ghi, 0);
         const int tiles = (nl + kTcCols - 1) / kTcCols + (nr + kTcCols - 1) / kTcCols;
         TimedLaunch t(tm, name, s);
-        const dim3 grid(npad_max / kTcRows, tiles, ns);
+        const dim3 grid(npad_max / kTcRows, tiles, nc);
         if (ghi - glo <= kTcNb)
             k_tc_update<true><<<grid, kTcUpdThreads, kTcUpdSmem, s>>>(A);
         else
             k_tc_update<false><<<grid, kTcUpdThreads, kTcUpdSmem, s>>>(A);
     };
-    // k_tc_panel: one cluster of kTcPanelCl CTAs per strip
+    // k_tc_panel: one cluster of kTcPanelCl CTAs per chain
     cudaLaunchAttribute pattr[1];
     pattr[0].id = cudaLaunchAttributeClusterDimension;
     pattr[0].val.clusterDim.x = kTcPanelCl;
     pattr[0].val.clusterDim.y = 1;
     pattr[0].val.clusterDim.z = 1;
     cudaLaunchConfig_t pcfg{};
-    pcfg.gridDim = dim3(ns * kTcPanelCl);
+    pcfg.gridDim = dim3(nc * kTcPanelCl);
     pcfg.blockDim = dim3(kTcPanelThreads);
     pcfg.dynamicSmemBytes = 0;
     pcfg.stream = s;
     pcfg.attrs = pattr;
     pcfg.numAttrs = 1;
     cudaError_t e = cudaSuccess;
-    for (int k = 0; k < g.Ny && e == cudaSuccess; ++k) {
-        for (int i = 0; i < ns && e == cudaSuccess; ++i) {
-            const StripDev& st = strips[i];
-            A.s[i].X = pool2 + st.fac + (int64_t)k * st.bs;
-            e = launch_slab_build<float2>(g, st, k, k > 0 ? pool2 + st.fac + (int64_t)(k - 1) * st.bs : nullptr,
-                                          st.ld, A.s[i].M, A.s[i].ldm, s, tm);
-            if (e == cudaSuccess) e = cudaMemsetAsync(A.s[i].kstep, 0xFF, (size_t)A.s[i].n * sizeof(int), s);
+    // step s: rows s (top chains) and N_y-1-s (bottom chains) up to the middle row t, then t,
+    // which needs both neighbours (the top chain's buffers)
+    const int t = (g.Ny - 1) / 2, nu = g.Ny - 1 - t;
+    for (int st = 0; st <= nu && e == cudaSuccess; ++st) {
+        for (int c = 0; c < nc; ++c) {
+            const StripDev& sd = strips[c / 2];
+            const bool up = c & 1, mid = st == nu;
+            TcStrip& S = A.s[c];
+            const bool live = up ? !mid : (mid || st < t);
+            S.n = live ? sd.W * g.Nz : 0;
+            S.k = up ? g.Ny - 1 - st : mid ? t : st;
+            if (!live) S.k = 0;
+            float2* X0 = pool2 + sd.fac;
+            S.X = X0 + (int64_t)S.k * sd.bs;
+            S.Xp = live && !up && S.k > 0 ? X0 + (int64_t)(S.k - 1) * sd.bs : nullptr;
+            S.Xn = live && (up || mid) && S.k + 1 < g.Ny ? X0 + (int64_t)(S.k + 1) * sd.bs : nullptr;
+        }
+        {
+            TimedLaunch t0(tm, "slab_build", s);
+            k_tc_build<<<sgrid, 256, 0, s>>>(g, A);
+            k_tc_dadd<<<dim3((5 * nmax + 63) / 64, nc), 64, 0, s>>>(g, A);
+            e = cudaGetLastError();
         }
         int sub = 0;
         for (int c0 = 0; c0 < nmax && e == cudaSuccess; c0 += kTcBig) {
@@ -668,13 +689,13 @@ cudaError_t launch_slab_factor_tc(const Geom& g, const StripDev* strips, int ns,
                 A.ghi = c1;
                 A.ulo = 0;
                 A.uhi = nmax;
-                k_tc_gather<<<dim3(((nmax - (c1 - c0)) * kTcBig + 255) / 256, ns), 256, 0, s>>>(A);
+                k_tc_gather<<<dim3(((nmax - (c1 - c0)) * kTcBig + 255) / 256, nc), 256, 0, s>>>(A);
                 update(c0, c1, 0, nmax, first, "slab_tc_update");
                 e = cudaGetLastError();
             }
         }
         if (e != cudaSuccess) break;
-        k_tc_pos<<<dim3(8, ns), 256, 0, s>>>(A);
+        k_tc_pos<<<dim3(8, nc), 256, 0, s>>>(A);
         {
             TimedLaunch t(tm, "slab_tc_store", s);
             k_tc_store<<<sgrid, 256, 0, s>>>(A);
