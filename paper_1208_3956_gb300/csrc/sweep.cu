@@ -253,7 +253,28 @@ __device__ __forceinline__ void dual_rows_r(const C (&sd)[NJ], const C (&su)[NJ]
     }
 }
 
-// The CTA is ceil(W/8) compute warps plus one producer warp.  The producer's
+// Compute warps of a tile of several right-hand sides (BT = 4, complex64).  Half of the warps run
+// the down chain of a step, half the up chain (a step's products are then one instruction
+// stream per chain, side by side), each half as (pair of right-hand sides) x (16 rows).  A lane
+// owns one row and half of the columns: 16-byte reads of the block's rows (conflict-free with
+// the +2 padding of the sweep layout), 16-byte reads of the two vectors that all lanes share,
+// and one exchange with the lane of the other column half, after which each of the two lanes
+// holds one right-hand side's sum.  Shared-memory reads bound a step's products (a warp-wide
+// 16-byte read takes 4 cycles, 2.3 when all lanes read one or two places: about 1220 cycles at
+// W = 45; 1330 measured).  With four lanes to a row and all four right-hand sides in a lane, as
+// for one right-hand side, the vectors were read four times over.  Lanes of 3 rows x 4
+// right-hand sides read less (900 cycles) but leave 8 warps to hide the latencies of 12, and
+// were slower (one P on 1055 rows, 4 and 32 right-hand sides: 8.0 and 20.5 ms against 6.4 and
+// 19.1 ms); so was one loop over all of a CTA's steps with a single copy of the products (4.8
+// against 4.2 ms at one right-hand side, 7.5 against 6.4 at four).  One P on 1055 rows, before
+// and after (with the output passes below): 4 right-hand sides 10.3 -> 6.4 ms, 8 (P = 75) 15.0
+// -> 8.5, 16 (P = 37) 20.6 -> 11.4, 32 (P = 18) 34.5 -> 19.1 ms.
+__host__ __device__ constexpr int panel_row_blocks(int W) { return (W + 15) / 16; }
+__host__ __device__ constexpr int chunk_threads(int W, int BT) {
+    return BT == 1 ? 32 * ((W + 7) / 8 + 1) : 32 * (4 * panel_row_blocks(W) + 1);
+}
+
+// The CTA is its compute warps plus one producer warp.  The producer's
 // lane 0 owns the TMA ring: it initialises the barriers, issues every bulk
 // copy, and right after each step's barrier refills the slots that step
 // consumed, while the compute warps already run the next step.  All factor
@@ -264,8 +285,10 @@ __device__ __forceinline__ void dual_rows_r(const C (&sd)[NJ], const C (&su)[NJ]
 // its group solves the group with those blocks already resident, the others
 // wait for their copies to land and exit.
 template <typename C, int NJ, int BT>
-__global__ void __launch_bounds__(288) k_sweep_chunk(SweepArgs A) {
+__global__ void __launch_bounds__(BT == 1 ? 288 : chunk_threads(4 * NJ, BT)) k_sweep_chunk(SweepArgs A) {
     using R = typename CT<C>::R;
+    constexpr bool kPanel = BT > 1;
+    static_assert(BT == 1 || BT == 4, "two pairs of right-hand sides to a panel tile");
     extern __shared__ __align__(128) unsigned char smem[];
     pdl_trigger();
     constexpr int LD = 4 * NJ + 2;
@@ -531,10 +554,9 @@ __global__ void __launch_bounds__(288) k_sweep_chunk(SweepArgs A) {
         const int ntask = A.has_prev ? nrow * 2 : 0;
         // the six rows of task t (unused ones zero), and the signs / switches they go with
         const bool on[6] = {has_above, has_below, fa0, fa1, fb0, fb1};
-        auto task_rows = [&](int task, C (&rw)[6][8]) {
+        auto row_ptrs = [&](int task, const C* (&rp)[6]) {
             const int kk = task >> 1, i = task & 1;
             const int col = 2 * A.sp.pdir + i, c = ps.xc[col];
-            const C* rp[6];
             if (kk < m) {
                 const int k = r0 + kk;
                 const int64_t ro = ps.fac + (int64_t)k * ps.bs + (int64_t)c * SLp;
@@ -549,6 +571,10 @@ __global__ void __launch_bounds__(288) k_sweep_chunk(SweepArgs A) {
                 rp[4] = NG > 1 ? reinterpret_cast<const C*>(A.GT2) + o2 : nullptr;
                 rp[5] = NG > 1 ? reinterpret_cast<const C*>(A.GB2) + o2 : nullptr;
             }
+        };
+        auto task_rows = [&](int task, C (&rw)[6][8]) {
+            const C* rp[6];
+            row_ptrs(task, rp);
 #pragma unroll
             for (int v = 0; v < 6; ++v)
 #pragma unroll
@@ -557,8 +583,23 @@ __global__ void __launch_bounds__(288) k_sweep_chunk(SweepArgs A) {
                     rw[v][q] = (rp[v] && on[v] && a < Wp) ? rp[v][a] : CT<C>::zero();
                 }
         };
-        C rw0[6][8];
-        if (ntask > 0) task_rows(imin(grp, ntask - 1), rw0);
+        // a panel tile's first rows only go to L2 here (its registers hold the sums of its
+        // right-hand sides later), one 128-byte line per lane
+        C rw0[kPanel ? 1 : 6][8];
+        if (ntask > 0) {
+            if constexpr (kPanel) {
+                for (int t0 = grp; t0 < ntask; t0 += ngrp) {
+                    const C* rp[6];
+                    row_ptrs(t0, rp);
+#pragma unroll
+                    for (int v = 0; v < 6; ++v)
+                        if (rp[v] && on[v] && lg * 128 < Wp * esz)
+                            asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char*>(rp[v]) + lg * 128));
+                }
+            } else {
+                task_rows(imin(grp, ntask - 1), rw0);
+            }
+        }
         pdl_wait();
         if (A.has_prev) {
             const C* Yp = reinterpret_cast<const C*>(A.pybuf);
@@ -578,8 +619,51 @@ __global__ void __launch_bounds__(288) k_sweep_chunk(SweepArgs A) {
                 const int task = imin(t0 + grp, ntask - 1);
                 const int kk = task >> 1, i = task & 1;
                 const int c = ps.xc[2 * A.sp.pdir + i];
-                if (t0 > 0) task_rows(task, rw0);   // the first task's rows were read before the wait
                 const bool srow = kk >= m;           // the separator row: x = y2_p - level-2 terms
+                if constexpr (kPanel) {
+                    const C* rp[6];
+                    row_ptrs(task, rp);
+                    C acc[BT];
+#pragma unroll
+                    for (int b = 0; b < BT; ++b) acc[b] = CT<C>::zero();
+#pragma unroll
+                    for (int v0 = 0; v0 < 6; v0 += 3) {   // three rows' loads in flight
+                        C rw[3][8];
+#pragma unroll
+                        for (int v = 0; v < 3; ++v)
+#pragma unroll
+                            for (int q = 0; q < 8; ++q) {
+                                const int a = lg + 8 * q;
+                                rw[v][q] = (rp[v0 + v] && on[v0 + v] && a < Wp) ? rp[v0 + v][a] : CT<C>::zero();
+                            }
+#pragma unroll
+                        for (int v = 0; v < 3; ++v)
+#pragma unroll
+                            for (int b = 0; b < BT; ++b)
+                                if (b < nb) {
+                                    C d = CT<C>::zero();
+#pragma unroll
+                                    for (int q = 0; q < 8; ++q)
+                                        d = cfma(rw[v][q], xv[((v0 + v) * BT + b) * 64 + lg + 8 * q], d);
+                                    acc[b] = cadd(acc[b], cscale(d, srow ? (R)-1 : sg[v0 + v]));
+                                }
+                    }
+#pragma unroll
+                    for (int b = 0; b < BT; ++b)
+                        if (b < nb) {
+#pragma unroll
+                            for (int o = 1; o <= 4; o <<= 1) {
+                                acc[b].x += __shfl_xor_sync(0xffffffffu, acc[b].x, o);
+                                acc[b].y += __shfl_xor_sync(0xffffffffu, acc[b].y, o);
+                            }
+                            if (live && lg == 0) {
+                                const C y = srow ? xv[(1 * BT + b) * 64 + c]
+                                                 : Yp[((int64_t)(b0 + b) * A.g.Ny + r0 + kk) * A.Wmax + c];
+                                xt[(kk * BT + b) * 2 + i] = cadd(y, acc[b]);
+                            }
+                        }
+                } else {
+                if (t0 > 0) task_rows(task, rw0);   // the first task's rows were read before the wait
                 for (int b = 0; b < nb; ++b) {
                     const C y = lg == 0 ? (srow ? xv[(1 * BT + b) * 64 + c]
                                                 : Yp[((int64_t)(b0 + b) * A.g.Ny + r0 + kk) * A.Wmax + c])
@@ -601,6 +685,7 @@ __global__ void __launch_bounds__(288) k_sweep_chunk(SweepArgs A) {
                         acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
                     }
                     if (live && lg == 0) xt[(kk * BT + b) * 2 + i] = cadd(y, acc);
+                }
                 }
             }
             asm volatile("bar.sync 1, %0;" ::"r"(ptid) : "memory");
@@ -627,12 +712,18 @@ __global__ void __launch_bounds__(288) k_sweep_chunk(SweepArgs A) {
     __syncthreads();
     // per-lane geometry
     const int w = tid >> 5, l = tid & 31;
-    const int row = w * 8 + (l >> 2);
-    const int g = l & 3;
+    const int nrb = panel_row_blocks(W);
+    const int g = kPanel ? l >> 4 : l & 3;                      // this lane's columns
+    const int row = kPanel ? (w % nrb) * 16 + (l & 15) : w * 8 + (l >> 2);
+    const bool upw = kPanel && w >= 2 * nrb;                    // panel: a warp of the up chain
+    const int bp = kPanel ? (w / nrb) & 1 : 0;                  // panel: pair of right-hand sides
+    const int ob = 2 * bp + g;                                  // panel: the right-hand side this lane finishes
     const bool rowok = compute && row < W;
+    const bool own = kPanel && rowok && ob < nb;
     const int rc = imin(row, W - 1);
-    const int lofs = rc * LD + g * NJ;     // this lane's run inside a block
-    const int vofs = g * NJ;               // ... and inside a vector
+    constexpr int kRun = kPanel ? 2 * NJ : NJ;                  // columns of a lane
+    const int lofs = rc * LD + g * kRun;   // this lane's run inside a block
+    const int vofs = g * kRun;             // ... and inside a vector
     const C csx_r = compute ? csx[rc] : CT<C>::zero();
     auto zr = [&](int k) -> C* { return zb + (k - r0) * BT * W; };   // row k, b = 0
     auto cpl = [&](int k) -> C { return cmul(csx_r, ccy[k - r0]); }; // C_k at this lane's row
@@ -653,11 +744,37 @@ __global__ void __launch_bounds__(288) k_sweep_chunk(SweepArgs A) {
     // barrier (the rows do not depend on the chain, so their shared-memory reads leave the
     // critical path of the slower FP64 products: 14 % faster; complex64 steps gained nothing
     // from it and read their rows in the step).
-    constexpr bool kPrefetch = sizeof(C) == sizeof(double2);
-    C rs_d[NJ], rs_u[NJ];
+    constexpr bool kPrefetch = !kPanel && sizeof(C) == sizeof(double2);
+    // panel: S-row . t for this lane's row and its pair of right-hand sides; returns the sum of
+    // right-hand side ob
+    auto prod = [&](const C* S, const C* t) -> C {
+        const C* sp = S + lofs;
+        const C* x0 = t + 2 * bp * 64 + vofs;
+        C a0 = CT<C>::zero(), a1 = CT<C>::zero(), c0 = CT<C>::zero(), c1 = CT<C>::zero();
+#pragma unroll
+        for (int j = 0; j < 2 * NJ; j += 2) {
+            C sv[2], xa[2], xb[2];
+            load_run2(sv, sp + j, 2);
+            load_run2(xa, x0 + j, 2);
+            load_run2(xb, x0 + 64 + j, 2);
+            a0 = cfma(sv[0], xa[0], a0);
+            c0 = cfma(sv[0], xb[0], c0);
+            a1 = cfma(sv[1], xa[1], a1);
+            c1 = cfma(sv[1], xb[1], c1);
+        }
+        const C a = cadd(a0, a1), c = cadd(c0, c1);
+        const C keep = g ? c : a, send = g ? a : c;
+        C r;
+        r.x = keep.x + __shfl_xor_sync(0xffffffffu, send.x, 16);
+        r.y = keep.y + __shfl_xor_sync(0xffffffffu, send.y, 16);
+        return r;
+    };
+    C rs_d[kPanel ? 1 : NJ], rs_u[kPanel ? 1 : NJ];
     bool have_rows = false;
     auto step2 = [&](const C* Sd, const C* td, const C* Su, const C* tu) {
-        if (compute) {
+        if constexpr (kPanel) {
+            return;
+        } else if (compute) {
             if (!have_rows) {
                 load_row<C, NJ>(rs_d, Sd + lofs);
                 load_row<C, NJ>(rs_u, Su + lofs);
@@ -668,11 +785,13 @@ __global__ void __launch_bounds__(288) k_sweep_chunk(SweepArgs A) {
     };
     // the next step's rows, read before this step's barrier
     auto prefetch = [&](const C* S1, const C* S2) {
-        if (compute) {
-            load_row<C, NJ>(rs_d, S1 + lofs);
-            load_row<C, NJ>(rs_u, S2 + lofs);
+        if constexpr (kPrefetch) {
+            if (compute) {
+                load_row<C, NJ>(rs_d, S1 + lofs);
+                load_row<C, NJ>(rs_u, S2 + lofs);
+            }
+            have_rows = true;
         }
-        have_rows = true;
     };
     // the blocks of a step with chains a (first in load order) and b, either may be off
     auto consume_ab = [&](bool a, bool b, const C*& Sa, const C*& Sb) {
@@ -684,7 +803,7 @@ __global__ void __launch_bounds__(288) k_sweep_chunk(SweepArgs A) {
         Sb = b ? (a ? S2 : S1) : nullptr;
     };
     const bool own1 = rowok && g == 0;                 // BT = 1: the lane that stores a row
-    auto owns = [&](int b) -> bool { return BT == 1 ? own1 : (b < nb && rowok && (b & 3) == g); };
+    auto owns = [&](int) -> bool { return own1; };
     C* const zl = zb + row;                            // this lane's entry of z-buffer row r0, b = 0
     const int zs = BT * W;                             // z-buffer stride between grid rows
     // One chain step of both halves, one code path for the forward, back and separator
@@ -702,6 +821,28 @@ __global__ void __launch_bounds__(288) k_sweep_chunk(SweepArgs A) {
     auto gstep = [&](auto&& pf, bool D, bool U, const C* S1, const C* S2, C* zd, C* zu, const C* znd, const C* znu,
                      C ckd, C cku, bool wvd, bool wvu, R az, R sv, R ez, R fc, bool pd = false, bool pu = false,
                      const C* pbase = nullptr, R ps = (R)1) -> bool {
+        if constexpr (kPanel) {   // each half of the warps its chain
+            if (compute && (upw ? U : D)) {
+                C* z = (upw ? zu : zd) + ob * W;
+                const C* zn = (upw ? znu : znd) + ob * W;
+                const C ck = upw ? cku : ckd;
+                const bool wv = upw ? wvu : wvd, pw = upw ? pu : pd;
+                const C pz = (own && az != (R)0) ? *z : CT<C>::zero();
+                const C pn = (own && wv && ez != (R)0) ? *zn : CT<C>::zero();
+                const C v = prod(upw && D ? S2 : S1, upw ? vin_u : vin_d);
+                if (own) {
+                    const C out = cadd(cscale(pz, az), cscale(v, sv));
+                    *z = out;
+                    const C vo = cadd(cscale(pn, ez), cscale(cmul(ck, out), fc));
+                    if (wv) (upw ? vout_u : vout_d)[ob * 64 + row] = vo;
+                    if (pw) {
+                        if (upw) pv_u[ob * 64 + row] = cadd(pbase ? pbase[ob * 64 + row] : CT<C>::zero(), cscale(vo, ps));
+                        else pv_d[ob * 64 + row] = cscale(vo, ps);
+                    }
+                }
+            }
+            return finish();
+        }
         C pzd[BT], pzu[BT], pnd[BT], pnu[BT];
 #pragma unroll
         for (int b = 0; b < BT; ++b) {
@@ -772,6 +913,18 @@ __global__ void __launch_bounds__(288) k_sweep_chunk(SweepArgs A) {
         const C* St = consume();
         step2(St, vin_d, St, vin_d);
         const C cd = cpl(t), cu = cpl(t + 1);
+        if constexpr (kPanel) {
+            if (compute && !upw) {
+                const C v = prod(St, vin_d);
+                if (own) {
+                    zr(t)[ob * W + row] = v;
+                    vout_d[ob * 64 + row] = cmul(cd, v);
+                    vout_u[ob * 64 + row] = cmul(cu, v);
+                    if (nd == 0) pv_d[ob * 64 + row] = cneg(cmul(cd, v));
+                    if (nu == 0) pv_u[ob * 64 + row] = csub(rsep[ob * 64 + row], cmul(cu, v));
+                }
+            }
+        } else {
 #pragma unroll
         for (int b = 0; b < BT; ++b)
             if (owns(b)) {
@@ -781,6 +934,7 @@ __global__ void __launch_bounds__(288) k_sweep_chunk(SweepArgs A) {
                 if (nd == 0) pv_d[b * 64 + row] = cneg(cmul(cd, vd[b]));              // t = r0
                 if (nu == 0) pv_u[b * 64 + row] = csub(rsep[b * 64 + row], cmul(cu, vd[b]));   // t = r1-1
             }
+        }
         if (!finish()) return;
     }
     // ---- outward back substitution: y_k = z_k - Sinv_k C y_inner
@@ -833,6 +987,20 @@ __global__ void __launch_bounds__(288) k_sweep_chunk(SweepArgs A) {
         const C *SA, *SB;
         consume_ab(has_below, has_above, SA, SB);
         step2(has_below ? SA : SB, has_below ? pv_u : pv_d, has_above ? SB : SA, has_above ? pv_d : pv_u);
+        if constexpr (kPanel) {
+            if (compute) {
+                const bool on_ = upw ? has_above : has_below;
+                const C v = on_ ? prod(upw ? SB : SA, upw ? pv_d : pv_u) : CT<C>::zero();
+                if (own) {
+                    const int sq = upw ? p - 1 : p;   // the separator
+                    if (on_) {
+                        if (NG > 1 && grp_of(sq) < 0) catomic_add(acc2 + a2idx(ob, -grp_of(sq) - 1) + row, v);
+                        else parts[pidx(ob, sq, upw ? 1 : 0) + row] = v;
+                    }
+                    (upw ? vout_u : vout_d)[ob * 64 + row] = v;
+                }
+            }
+        } else {
 #pragma unroll
         for (int b = 0; b < BT; ++b)
             if (b < nb && rowok && (b & 3) == g) {
@@ -850,11 +1018,26 @@ __global__ void __launch_bounds__(288) k_sweep_chunk(SweepArgs A) {
                 vout_d[b * 64 + row] = has_below ? vd[b] : CT<C>::zero();
                 vout_u[b * 64 + row] = has_above ? vu[b] : CT<C>::zero();
             }
+        }
         if (!finish()) return;
     }
     if (NG > 1) {
         // ---- the chunk's contributions to the level-2 right-hand sides below (dn) and above
         // (up) its group: Q2L/Q2U of separator p times A_p, of separator p-1 times B_{p-1}
+        const int gg0 = q2dnA || q2upA ? grp_of(p) : grp_of(imax(p - 1, 0));
+        auto contrib_panel = [&](bool a, bool b, int r) {   // each half of the warps one separator's term
+            if (!a && !b) return;
+            const C *SA, *SB;
+            consume_ab(a, b, SA, SB);
+            if (compute && (upw ? b : a)) {
+                const C v = prod(upw ? SB : SA, upw ? vin_u : vin_d);
+                if (own) catomic_add(acc2 + a2idx(ob, r) + row, v);
+            }
+        };
+        if constexpr (kPanel) {
+            contrib_panel(q2dnA, q2dnB, gg0);
+            contrib_panel(q2upA, q2upB, gg0 - 1);
+        } else {
         C dn[BT], up[BT];
         auto contrib = [&](bool a, bool b, C (&out)[BT]) {
 #pragma unroll
@@ -879,6 +1062,7 @@ __global__ void __launch_bounds__(288) k_sweep_chunk(SweepArgs A) {
                 if (q2dnA || q2dnB) catomic_add(acc2 + a2idx(b, gg) + row, dn[b]);
                 if (q2upA || q2upB) catomic_add(acc2 + a2idx(b, gg - 1) + row, up[b]);
             }
+        }
         if (!finish()) return;
         // release: this CTA's parts and contributions (ordered before by the barrier)
         if (tid == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(cnt + NG) : "memory");
@@ -941,6 +1125,21 @@ __global__ void __launch_bounds__(288) k_sweep_chunk(SweepArgs A) {
             const C *Se, *Sf;
             consume_ab(he, hf, Se, Sf);
             step2(he ? Se : Sf, he ? vin_d : vin_u, hf ? Sf : Se, hf ? vin_u : vin_d);
+            if constexpr (kPanel) {
+                const bool on_ = upw ? hf : he;
+                const C v = (compute && on_) ? prod(upw ? Sf : Se, upw ? vin_u : vin_d) : CT<C>::zero();
+                if (upw && own) vout_u[ob * 64 + row] = v;   // to the lane that sums both terms
+                __syncthreads();
+                if (!upw && own) {
+                    C* zp = zq(tq) + ob * W + row;
+                    const C x = csub(csub(*zp, v), vout_u[ob * 64 + row]);
+                    *zp = x;
+                    vout_d[ob * 64 + row] = x;
+                    vout_u[ob * 64 + row] = x;
+                    if (tq == 0) pv_d[ob * 64 + row] = x;
+                    if (tq == n - 1) pv_u[ob * 64 + row] = x;
+                }
+            } else {
 #pragma unroll
             for (int b = 0; b < BT; ++b)
                 if (b < nb && rowok && (b & 3) == g) {
@@ -954,6 +1153,7 @@ __global__ void __launch_bounds__(288) k_sweep_chunk(SweepArgs A) {
                     if (tq == 0) pv_d[b * 64 + row] = x;        // x_0
                     if (tq == n - 1) pv_u[b * 64 + row] = x;    // x_{n-1}
                 }
+            }
             if (!finish()) return false;
         }
         // back: x_i = z_i - F_i x_inner, down i = tq-1..0, up i = tq+1..n-1; the last
@@ -1196,6 +1396,190 @@ __global__ void __launch_bounds__(256, 2) k_sweep_output(OutArgs O, const C* __r
     }
 }
 
+// The same pass for several right-hand sides.  A work item is a chunk of a strip with up to kTB
+// right-hand sides, so that the spike rows are read once for all of them: a group of 8 lanes
+// holds the two spike rows of two adjacent outputs (16-byte loads) and multiplies them, four
+// right-hand sides at a time, with the separator values in shared memory; the 2 x 8 sums
+// (right-hand sides x components) are folded over the 8 lanes, each of which finishes and
+// writes one component of either output.  With the right-hand sides in the outer loop, as for
+// one, the spike rows were read once per right-hand side and the passes held up a panel's sweep:
+// 23.2 ms of output passes beside 34 ms of strip solves per application of P at 32
+// right-hand sides on 1055 rows, 8.9 ms now.
+template <typename C>
+struct Pair2 { C a, b; };
+__device__ __forceinline__ Pair2<float2> load_pair(const float2* p) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    return {make_float2(q.x, q.y), make_float2(q.z, q.w)};
+}
+__device__ __forceinline__ Pair2<double2> load_pair(const double2* p) { return {p[0], p[1]}; }
+constexpr int kPanelOut = 16;   // kTB
+
+template <typename C>
+__global__ void __launch_bounds__(256, 2) k_sweep_output_panel(OutArgs O, const C* __restrict__ GT,
+                                                               const C* __restrict__ GB, const C* __restrict__ GT2,
+                                                               const C* __restrict__ GB2) {
+    using R = typename CT<C>::R;
+    constexpr int kTB = kPanelOut, BT = 4;
+    __shared__ __align__(16) C xsv[2][kTB][64];     // final values of the separators above / below, zero beyond W
+    __shared__ __align__(16) C xl[2][BT][64];       // level-2 values above / below a separator's group
+    const int ntile = (O.B + kTB - 1) / kTB;
+    const int nitem = O.g.P * O.nstrip * ntile;
+    const int tid = threadIdx.x, g = tid & 7, grp = tid >> 3, ngrp = blockDim.x >> 3;
+    // this lane's entries of the two spike rows of an output (null: absent), W entries a row
+    auto load_rows = [&](const C* ra, const C* rb, int W, Pair2<C> (&sa)[4], Pair2<C> (&sb)[4]) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int a = 2 * g + 16 * i;
+            sa[i].a = sa[i].b = sb[i].a = sb[i].b = CT<C>::zero();
+            if (ra && a < W) sa[i] = load_pair(ra + a);
+            if (rb && a < W) sb[i] = load_pair(rb + a);
+            if (a + 1 >= W) sa[i].b = sb[i].b = CT<C>::zero();   // the rows' padding
+        }
+    };
+    // sums of v (4 right-hand sides x 2 components) over the 8 lanes: lane g gets component
+    // g & 1 of right-hand side g >> 1
+    auto fold = [&](const C (&acc)[BT]) -> R {
+        R v[8], w[4], u[2];
+#pragma unroll
+        for (int b = 0; b < BT; ++b) { v[2 * b] = acc[b].x; v[2 * b + 1] = acc[b].y; }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            w[i] = ((g & 4) ? v[i + 4] : v[i]) + __shfl_xor_sync(0xffffffffu, (g & 4) ? v[i] : v[i + 4], 4);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            u[i] = ((g & 2) ? w[i + 2] : w[i]) + __shfl_xor_sync(0xffffffffu, (g & 2) ? w[i] : w[i + 2], 2);
+        return ((g & 1) ? u[1] : u[0]) + __shfl_xor_sync(0xffffffffu, (g & 1) ? u[0] : u[1], 1);
+    };
+    const int gb = g >> 1, gc = g & 1;   // the right-hand side and component this lane finishes
+    for (int item = blockIdx.x; item < nitem; item += gridDim.x) {   // (chunk, strip, right-hand sides)
+        __syncthreads();   // the shared vectors of the previous item are consumed
+        const int p = item % O.g.P;
+        const int j = O.jlo + (item / O.g.P) % O.nstrip;
+        const int b0 = (item / (O.g.P * O.nstrip)) * kTB;
+        const int nb = imin(kTB, O.B - b0);
+        const StripDev& st = O.g.strips[j];
+        const int W = st.W, SL = spld(W);
+        const int P = O.g.P, NG = O.g.G;
+        const int off = st.lo - st.lpml;
+        const int olo = imax(st.olo[O.dir] - off, 0), ohi = imin(st.ohi[O.dir] - off, W - 1);
+        const int nout = ohi - olo + 1;
+        if (nout <= 0) continue;   // uniform
+        const int4 m0 = O.g.cmeta[2 * p], m1 = O.g.cmeta[2 * p + 1];
+        const int r0 = m0.x, r1 = m0.y, m = r1 - r0;
+        const C* Y = reinterpret_cast<const C*>(O.ybuf) + (int64_t)j * O.ystride;
+        auto yr = [&](int b, int k) { return Y + ((int64_t)(b0 + b) * O.g.Ny + k) * O.Wmax; };
+        const bool above = p > 0, below = p < P - 1;
+        // ---- the separators' values as the chain kernel left them ...
+        for (int o = tid; o < 2 * kTB * 64; o += blockDim.x) {
+            const int c = o & 63, b = (o >> 6) % kTB, side = o / (64 * kTB);
+            const bool have = (side == 0 ? above : below) && b < nb && c < W;
+            xsv[side][b][c] = have ? yr(b, side == 0 ? r0 - 1 : r1)[c] : CT<C>::zero();
+        }
+        // ... and, for grouped ones, x_q = y2_q - GT2_q x2_above - GB2_q x2_below
+        for (int side = 0; side < 2; ++side) {
+            const int sg = side == 0 ? m0.z : m0.w;
+            const bool have = side == 0 ? above : below;
+            const bool up = have && sg > 0, dn = have && sg >= 0 && sg < NG - 1;
+            if (!up && !dn) continue;   // uniform
+            const int64_t o2 = st.red + (int64_t)(side == 0 ? p - 1 : p) * st.bs;
+            for (int q0 = 0; q0 < nb; q0 += BT) {
+                __syncthreads();
+                for (int o = tid; o < 2 * BT * 64; o += blockDim.x) {
+                    const int c = o & 63, b = (o >> 6) % BT, lv = o / (64 * BT);
+                    const int k = lv == 0 ? (side == 0 ? m1.x : m1.z) : (side == 0 ? m1.y : m1.w);
+                    xl[lv][b][c] = ((lv == 0 ? up : dn) && q0 + b < nb && c < W) ? yr(q0 + b, k)[c] : CT<C>::zero();
+                }
+                __syncthreads();
+                for (int c0 = 0; c0 < W; c0 += ngrp) {   // uniform trip count: every lane shuffles
+                    const int c = c0 + grp, cc = imin(c, W - 1);
+                    Pair2<C> sa[4], sb[4];
+                    load_rows(up ? GT2 + o2 + (int64_t)cc * SL : nullptr, dn ? GB2 + o2 + (int64_t)cc * SL : nullptr, W,
+                              sa, sb);
+                    C acc[BT];
+#pragma unroll
+                    for (int b = 0; b < BT; ++b) acc[b] = CT<C>::zero();
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+#pragma unroll
+                        for (int b = 0; b < BT; ++b) {
+                            const int o = 2 * g + 16 * i;
+                            const Pair2<C> x = load_pair(&xl[0][b][o]), y = load_pair(&xl[1][b][o]);
+                            acc[b] = cfma(sa[i].a, x.a, acc[b]);
+                            acc[b] = cfma(sa[i].b, x.b, acc[b]);
+                            acc[b] = cfma(sb[i].a, y.a, acc[b]);
+                            acc[b] = cfma(sb[i].b, y.b, acc[b]);
+                        }
+                    }
+                    const R sum = fold(acc);
+                    if (c < W && q0 + gb < kTB) reinterpret_cast<R*>(&xsv[side][q0 + gb][c])[gc] -= sum;
+                }
+            }
+        }
+        __syncthreads();
+        auto at = [&](int b, int k, int c) { return ((int64_t)(b0 + b) * O.g.Ny + k) * O.g.Nx + off + c; };
+        if (below)   // the separator row below the chunk: its final value
+            for (int o = tid; o < nb * nout; o += blockDim.x) {
+                const int b = o / nout, c = olo + o % nout;
+                double2 v = to_d2(xsv[1][b][c]);
+                if (O.base) v = cadd(v, O.base[at(b, r1, c)]);
+                O.dst[at(b, r1, c)] = v;
+            }
+        // ---- x_k = y_k - GT_p(k) x_{p-1} - GB_p(k) x_p, two adjacent outputs to a group
+        const int ntask = m * nout;
+        for (int t0 = 0; t0 < ntask; t0 += 2 * ngrp) {   // uniform trip count: every lane shuffles
+            int k[2], c[2];
+            bool live[2];
+            Pair2<C> sa[2][4], sb[2][4];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int t = t0 + 2 * grp + u, tc = imin(t, ntask - 1);
+                live[u] = t < ntask;
+                k[u] = r0 + tc / nout;
+                c[u] = olo + tc % nout;
+                const int64_t ro = st.fac + (int64_t)k[u] * st.bs + (int64_t)c[u] * SL;
+                load_rows(above ? GT + ro : nullptr, below ? GB + ro : nullptr, W, sa[u], sb[u]);
+            }
+            for (int q0 = 0; q0 < nb; q0 += BT) {
+                const int bb = imin(q0 + gb, nb - 1);
+                R y[2];
+                double bv[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    y[u] = reinterpret_cast<const R*>(yr(bb, k[u]) + c[u])[gc];
+                    bv[u] = O.base ? reinterpret_cast<const double*>(O.base + at(bb, k[u], c[u]))[gc] : 0.0;
+                }
+                C acc[2][BT];
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+#pragma unroll
+                    for (int b = 0; b < BT; ++b) acc[u][b] = CT<C>::zero();
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if (16 * i >= W) continue;   // uniform
+#pragma unroll
+                    for (int b = 0; b < BT; ++b) {
+                        const int o = 2 * g + 16 * i;
+                        const Pair2<C> x = load_pair(&xsv[0][q0 + b][o]), z = load_pair(&xsv[1][q0 + b][o]);
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            acc[u][b] = cfma(sa[u][i].a, x.a, acc[u][b]);
+                            acc[u][b] = cfma(sa[u][i].b, x.b, acc[u][b]);
+                            acc[u][b] = cfma(sb[u][i].a, z.a, acc[u][b]);
+                            acc[u][b] = cfma(sb[u][i].b, z.b, acc[u][b]);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const R sum = fold(acc[u]);
+                    if (live[u] && q0 + gb < nb)
+                        reinterpret_cast<double*>(O.dst + at(bb, k[u], c[u]))[gc] = (double)(y[u] - sum) + bv[u];
+                }
+            }
+        }
+    }
+}
+
 // ------------------------------------------------------------------ host
 // Bytes of the separator-parts region of a strip solve ([B][P-1][kParts][Wmax]); the
 // level-2 accumulators ([B][G-1][Wmax], sized for G - 1 <= P) follow it.
@@ -1246,7 +1630,10 @@ template <typename C>
 static bool plan(const StripDev& st, int zrows, int B, int& Bt, int& ring, size_t& smem) {
     const size_t budget = 220 * 1024;
     const uint32_t slot = (uint32_t)(st.bs * sizeof(C));
-    for (Bt = (B > 1 ? 4 : 1); Bt >= 1; Bt -= 3) {   // tiles of 4 right-hand sides, or 1
+    // tiles of 4 right-hand sides in complex64, or 1.  Complex128 is bound by the FP64 pipe of the
+    // SMs that run a strip solve, so its right-hand sides go to separate CTAs (511 x 511 grid, two
+    // right-hand sides: 18.9 ms for one P in one 4-wide tile, 11.5 ms in two tiles)
+    for (Bt = (B > 1 && sizeof(C) == sizeof(float2) ? 4 : 1); Bt >= 1; Bt -= 3) {
         for (ring = kMaxRing; ring >= 4; --ring) {
             smem = sweep_smem(ring, slot, zrows, Bt, st.W, (int)sizeof(C)).total;
             if (smem <= budget) return true;
@@ -1265,14 +1652,18 @@ bool strip_solve_fits(const StripDev& st, int zrows, size_t esize) {
 // Shared-memory limit of every strip-solve instantiation (this also loads the module).
 template <typename C>
 static cudaError_t chunk_kernel_attrs() {
-    for (auto fn : {k_sweep_chunk<C, 8, 1>, k_sweep_chunk<C, 10, 1>, k_sweep_chunk<C, 12, 1>,
-                    k_sweep_chunk<C, 14, 1>, k_sweep_chunk<C, 16, 1>, k_sweep_chunk<C, 8, 4>,
-                    k_sweep_chunk<C, 10, 4>, k_sweep_chunk<C, 12, 4>, k_sweep_chunk<C, 14, 4>,
-                    k_sweep_chunk<C, 16, 4>}) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    auto set = [&](void (*fn)(SweepArgs)) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+    };
+    for (auto fn : {k_sweep_chunk<C, 8, 1>, k_sweep_chunk<C, 10, 1>, k_sweep_chunk<C, 12, 1>, k_sweep_chunk<C, 14, 1>,
+                    k_sweep_chunk<C, 16, 1>})
+        set(fn);
+    if constexpr (sizeof(C) == sizeof(float2))
+        for (auto fn : {k_sweep_chunk<C, 8, 4>, k_sweep_chunk<C, 10, 4>, k_sweep_chunk<C, 12, 4>,
+                        k_sweep_chunk<C, 14, 4>, k_sweep_chunk<C, 16, 4>})
+            set(fn);
+    return e;
 }
 
 cudaError_t preload_sweep_kernels() {
@@ -1281,6 +1672,7 @@ cudaError_t preload_sweep_kernels() {
     cudaFuncAttributes fa;
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_sweep_output<float2>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_sweep_output<double2>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_sweep_output_panel<float2>);
     return e;
 }
 
@@ -1320,7 +1712,8 @@ cudaError_t launch_strip_solve(const Geom& g, int j, const StripDev& st, const S
     cudaError_t err;
     {
         void (*kfn)(SweepArgs) = nullptr;
-#define HELM_CHUNK_FN(NJ) kfn = Bt == 1 ? k_sweep_chunk<C, NJ, 1> : k_sweep_chunk<C, NJ, 4>
+        constexpr int kBt = sizeof(C) == sizeof(float2) ? 4 : 1;
+#define HELM_CHUNK_FN(NJ) kfn = Bt == 1 ? k_sweep_chunk<C, NJ, 1> : k_sweep_chunk<C, NJ, kBt>
         switch (st.nj) {
             case 8: HELM_CHUNK_FN(8); break;
             case 10: HELM_CHUNK_FN(10); break;
@@ -1330,7 +1723,7 @@ cudaError_t launch_strip_solve(const Geom& g, int j, const StripDev& st, const S
         }
 #undef HELM_CHUNK_FN
         // compute warps + the producer warp; with separator groups one more CTA for level 2
-        const cudaLaunchConfig_t cfg = config(dim3(g.P + (g.G > 1 ? 1 : 0), ntile), 32 * ((st.W + 7) / 8 + 1), smem);
+        const cudaLaunchConfig_t cfg = config(dim3(g.P + (g.G > 1 ? 1 : 0), ntile), chunk_threads(st.W, Bt), smem);
         TimedLaunch t(tm, "sweep_chunk", s);
         err = cudaLaunchKernelEx(&cfg, kfn, A);
     }
@@ -1342,10 +1735,17 @@ template <typename C>
 cudaError_t launch_outputs(const OutArgs& O, void* const* pool, cudaStream_t s, KernelTimer* tm) {
     if (O.nstrip <= 0) return cudaSuccess;
     TimedLaunch t(tm, "sweep_output", s);
-    const int nitem = O.g.P * O.nstrip * ((O.B + O.Bt - 1) / O.Bt);
+    const C *GT = (const C*)pool[1], *GB = (const C*)pool[2], *GT2 = (const C*)pool[6], *GB2 = (const C*)pool[7];
+    // several right-hand sides in complex64: the spike rows once for all of them (complex128 is
+    // bound by the FP64 pipe, which a padded group of four right-hand sides would waste)
+    const bool panel = O.Bt > 1 && sizeof(C) == sizeof(float2);
+    const int bt = panel ? kPanelOut : O.Bt;
+    const int nitem = O.g.P * O.nstrip * ((O.B + bt - 1) / bt);
     const int grid = O.maxcta > 0 ? imin(nitem, O.maxcta) : nitem;
-    k_sweep_output<C><<<grid, 256, 0, s>>>(O, (const C*)pool[1], (const C*)pool[2], (const C*)pool[6],
-                                         (const C*)pool[7]);
+    if constexpr (sizeof(C) == sizeof(float2)) {
+        if (panel) k_sweep_output_panel<C><<<grid, 256, 0, s>>>(O, GT, GB, GT2, GB2);
+    }
+    if (!panel) k_sweep_output<C><<<grid, 256, 0, s>>>(O, GT, GB, GT2, GB2);
     return cudaGetLastError();
 }
 
