@@ -203,9 +203,12 @@ __global__ void k_multidot(const double2* __restrict__ V, int64_t vstride, const
     }
 }
 
-// out[b*nv+i] = sum over blocks, fixed order (deterministic)
+// out[b*nv+i] = sum over blocks, fixed order (deterministic); with coef, also coef[b*nv+i] = -out
+// where column b is active (act[b] != 0), else 0: the update coefficients of the
+// orthogonalisation, without a trip through the host
 __global__ void k_reduce_partials(const double2* __restrict__ partial, int nblk, int count,
-                                  double2* __restrict__ out) {
+                                  double2* __restrict__ out, double2* __restrict__ coef,
+                                  const double* __restrict__ act, int nv) {
     const int id = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (id >= count) return;
@@ -219,11 +222,15 @@ __global__ void k_reduce_partials(const double2* __restrict__ partial, int nblk,
         re += __shfl_xor_sync(0xffffffffu, re, o);
         im += __shfl_xor_sync(0xffffffffu, im, o);
     }
-    if (lane == 0) out[id] = make_double2(re, im);
+    if (lane == 0) {
+        out[id] = make_double2(re, im);
+        if (coef) coef[id] = act[id / nv] != 0.0 ? make_double2(-re, -im) : make_double2(0.0, 0.0);
+    }
 }
 
 cudaError_t launch_multidot(const double2* V, int64_t vstride, const double2* w, int nv, int B, int64_t N,
-                            double2* partial, int nblk, double2* out, cudaStream_t s, KernelTimer* tm) {
+                            double2* partial, int nblk, double2* out, cudaStream_t s, KernelTimer* tm,
+                            double2* coef, const double* act) {
     {
         TimedLaunch t(tm, "krylov_dot", s);
         k_multidot<<<dim3(nblk, nv, B), 256, 0, s>>>(V, vstride, w, nv, B, N, partial);
@@ -232,7 +239,7 @@ cudaError_t launch_multidot(const double2* V, int64_t vstride, const double2* w,
     if (err != cudaSuccess) return err;
     const int count = nv * B;
     TimedLaunch t(tm, "krylov_reduce", s);
-    k_reduce_partials<<<(count + 7) / 8, 256, 0, s>>>(partial, nblk, count, out);
+    k_reduce_partials<<<(count + 7) / 8, 256, 0, s>>>(partial, nblk, count, out, coef, act, nv);
     return cudaGetLastError();
 }
 

@@ -114,6 +114,8 @@ struct helm_dd {
     void* noalloc_base = nullptr;   // device address of the no-allocation scratch array
     // workspaces
     struct Ws { void* p = nullptr; size_t bytes = 0; };
+    void* host_small = nullptr;     // page-locked, host_small_bytes: the Krylov loop's small transfers
+    size_t host_small_bytes = 0;
     Ws ws_V, ws_G, ws_Y, ws_parts, ws_io_in, ws_io_out, ws_io_aux, ws_kry, ws_small, ws_grad, ws_red;
     // interface lines of the reduced space (Section 2.3): padded columns beta_j+1, beta_j+2
     std::vector<int> icols;
@@ -154,6 +156,19 @@ void ws_free(helm_dd::Ws& w) {
     if (w.p) cudaFree(w.p);
     w.p = nullptr;
     w.bytes = 0;
+}
+
+// Page-locked host memory of a handle, grown when needed (pending copies use the old one until
+// the stream is idle).
+helm_status host_reserve(helm_dd* h, size_t bytes) {
+    if (h->host_small_bytes >= bytes) return HELM_OK;
+    CK(h, cudaStreamSynchronize(h->stream));
+    if (h->host_small) cudaFreeHost(h->host_small);
+    h->host_small = nullptr;
+    h->host_small_bytes = 0;
+    CK(h, cudaMallocHost(&h->host_small, bytes));
+    h->host_small_bytes = bytes;
+    return HELM_OK;
 }
 
 // complex128 device fields are read with 16-byte accesses
@@ -1371,7 +1386,7 @@ helm_status dev_gmres(helm_dd* h, const KrylovOp& op, const double2* F, double2*
     // Krylov storage: V_0..V_m, Z_0..Z_{m-1} (flexible only), W
     if ((s = ws_reserve(h, h->ws_kry, (size_t)(flex ? 2 * m + 2 : m + 2) * vb)) != HELM_OK) return s;
     const int nblk = 304;
-    const size_t small = (size_t)B * (m + 2) * nblk * sizeof(double2) + (size_t)4 * B * (m + 2) * sizeof(double2);
+    const size_t small = (size_t)B * (m + 2) * nblk * sizeof(double2) + (size_t)6 * B * (m + 2) * sizeof(double2);
     if ((s = ws_reserve(h, h->ws_small, small)) != HELM_OK) return s;
     double2* V = (double2*)h->ws_kry.p;
     const int64_t vs = (int64_t)B * NV;   // stride between Krylov vectors (elements)
@@ -1379,14 +1394,19 @@ helm_status dev_gmres(helm_dd* h, const KrylovOp& op, const double2* F, double2*
     double2* Wv = flex ? Z + (int64_t)m * vs : V + (int64_t)(m + 1) * vs;
     double2* partial = (double2*)h->ws_small.p;
     double2* dres = partial + (size_t)B * (m + 2) * nblk;
-    double2* dcoef = dres + (size_t)B * (m + 2);
+    double2* dcoef = dres + (size_t)3 * B * (m + 2);   // dres: the two passes' products, then the norms
     double* dscale = (double*)(dcoef + (size_t)B * (m + 2));
-    std::vector<double2> hres(B * (m + 2)), hcoef(B * (m + 2));
-    std::vector<double> hscale(B);
+    // page-locked host side of the small transfers (kept with the handle): a pageable copy of a few
+    // values costs a staging step and a synchronisation of its own
+    const size_t hres_n = (size_t)3 * B * (m + 2), hcoef_n = (size_t)B * (m + 2);
+    if ((s = host_reserve(h, (hres_n + hcoef_n) * sizeof(double2) + B * sizeof(double))) != HELM_OK) return s;
+    double2* hres = (double2*)h->host_small;
+    double2* hcoef = hres + hres_n;
+    double* hscale = (double*)(hcoef + hcoef_n);
 
     auto norms = [&](const double2* X, std::vector<double>& nrm) -> helm_status {
         CK(h, launch_multidot(X, 0, X, 1, B, NV, partial, nblk, dres, h->stream, &h->timer));
-        CK(h, cudaMemcpyAsync(hres.data(), dres, B * sizeof(double2), cudaMemcpyDeviceToHost, h->stream));
+        CK(h, cudaMemcpyAsync(hres, dres, B * sizeof(double2), cudaMemcpyDeviceToHost, h->stream));
         CK(h, cudaStreamSynchronize(h->stream));
         nrm.resize(B);
         for (int b = 0; b < B; ++b) nrm[b] = sqrt(std::max(hres[b].x, 0.0));
@@ -1428,33 +1448,35 @@ helm_status dev_gmres(helm_dd* h, const KrylovOp& op, const double2* F, double2*
             g[(size_t)b * (m + 1)] = beta[b];
         }
         if (!any || ++guard > 100000) break;
-        CK(h, cudaMemcpyAsync(dscale, hscale.data(), B * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+        CK(h, cudaMemcpyAsync(dscale, hscale, B * sizeof(double), cudaMemcpyHostToDevice, h->stream));
         CK(h, launch_scale(V, V, dscale, B, NV, h->stream, &h->timer));
         for (int i = 0; i < m; ++i) {
             double2* Vi = V + (int64_t)i * vs;
             double2* Zi = Z + (int64_t)i * vs;
             if (flex && (s = op.precond(Vi, Zi, B)) != HELM_OK) return s;
             if ((s = op.residual(Zi, nullptr, Wv, B)) != HELM_OK) return s;
-            // CGS2
-            std::vector<cd> hcol((size_t)B * (i + 1), 0.0);
+            // CGS2: both passes and the norm queued together, the update coefficients formed on the device
+            // (dscale holds the columns' scale factors of this step: zero where a column is done), one
+            // trip to the host a step.  Three trips a step, the coefficients through the host: 3.34 ms a
+            // solve on 127 x 127 (7 iterations), now 3.15 ms.
+            const size_t nh = (size_t)B * (i + 1);
             for (int pass = 0; pass < 2; ++pass) {
-                CK(h, launch_multidot(V, vs, Wv, i + 1, B, NV, partial, nblk, dres, h->stream, &h->timer));
-                CK(h, cudaMemcpyAsync(hres.data(), dres, (size_t)B * (i + 1) * sizeof(double2),
-                                      cudaMemcpyDeviceToHost, h->stream));
-                CK(h, cudaStreamSynchronize(h->stream));
-                for (int b = 0; b < B; ++b)
-                    for (int k = 0; k <= i; ++k) {
-                        const double2 v = hres[(size_t)b * (i + 1) + k];
-                        const cd hv = active[b] ? cd(v.x, v.y) : cd(0.0);
-                        hcol[(size_t)b * (i + 1) + k] += hv;
-                        hcoef[(size_t)b * (i + 1) + k] = make_double2(-hv.real(), -hv.imag());
-                    }
-                CK(h, cudaMemcpyAsync(dcoef, hcoef.data(), (size_t)B * (i + 1) * sizeof(double2),
-                                      cudaMemcpyHostToDevice, h->stream));
+                CK(h, launch_multidot(V, vs, Wv, i + 1, B, NV, partial, nblk, dres + pass * nh, h->stream, &h->timer,
+                                      dcoef, dscale));
                 CK(h, launch_multi_axpy(Wv, V, vs, dcoef, i + 1, B, NV, h->stream, &h->timer));
             }
-            std::vector<double> hn;
-            if ((s = norms(Wv, hn)) != HELM_OK) return s;
+            CK(h, launch_multidot(Wv, 0, Wv, 1, B, NV, partial, nblk, dres + 2 * nh, h->stream, &h->timer));
+            CK(h, cudaMemcpyAsync(hres, dres, (2 * nh + B) * sizeof(double2), cudaMemcpyDeviceToHost, h->stream));
+            CK(h, cudaStreamSynchronize(h->stream));
+            std::vector<cd> hcol(nh, 0.0);
+            std::vector<double> hn(B);
+            for (int b = 0; b < B; ++b) {
+                hn[b] = sqrt(std::max(hres[2 * nh + b].x, 0.0));
+                for (int k = 0; k <= i && active[b]; ++k) {
+                    const size_t o = (size_t)b * (i + 1) + k;
+                    hcol[o] = cd(hres[o].x, hres[o].y) + cd(hres[nh + o].x, hres[nh + o].y);
+                }
+            }
             bool still = false;
             for (int b = 0; b < B; ++b) {
                 if (!active[b]) { hscale[b] = 0.0; continue; }
@@ -1495,7 +1517,7 @@ helm_status dev_gmres(helm_dd* h, const KrylovOp& op, const double2* F, double2*
                 still = still || active[b];
             }
             if (!still || i == m - 1) break;
-            CK(h, cudaMemcpyAsync(dscale, hscale.data(), B * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+            CK(h, cudaMemcpyAsync(dscale, hscale, B * sizeof(double), cudaMemcpyHostToDevice, h->stream));
             CK(h, launch_scale(V + (int64_t)(i + 1) * vs, Wv, dscale, B, NV, h->stream, &h->timer));
         }
         // x += Z y,  H y = g (upper triangular, per column)
@@ -1516,7 +1538,7 @@ helm_status dev_gmres(helm_dd* h, const KrylovOp& op, const double2* F, double2*
             }
         }
         if (kmax > 0) {
-            CK(h, cudaMemcpyAsync(dcoef, hcoef.data(), (size_t)B * kmax * sizeof(double2), cudaMemcpyHostToDevice,
+            CK(h, cudaMemcpyAsync(dcoef, hcoef, (size_t)B * kmax * sizeof(double2), cudaMemcpyHostToDevice,
                                   h->stream));
             CK(h, launch_multi_axpy(U, Z, vs, dcoef, kmax, B, NV, h->stream, &h->timer));
         }
@@ -2106,6 +2128,7 @@ void helm_dd_destroy(helm_dd* h) {
     cudaFree(h->d_ct);
     cudaFree(h->d_slab_sxz);
     cudaFree(h->d_slab_scratch);
+    if (h->host_small) cudaFreeHost(h->host_small);
     cudaFree(h->d_counters);
     cudaFree(h->d_icols);
     cudaFree(h->d_rab);

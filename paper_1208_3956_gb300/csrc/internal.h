@@ -216,9 +216,11 @@ cudaError_t launch_stencil(const Geom& g, const double2* u, const double2* f, do
                            cudaStream_t s, KernelTimer* tm);
 cudaError_t launch_copy_cols(const double2* src, double2* dst, int B, int Nx, int Ny, int Nz, int xlo, int xhi,
                              cudaStream_t s, KernelTimer* tm);
+// (coef, if given: -h[b][i] where act[b] != 0, else 0)
 // partial[b][i][blk] for h[b][i] = sum_n conj(V_i[b][n]) w[b][n]; V_i at V + i*vstride
 cudaError_t launch_multidot(const double2* V, int64_t vstride, const double2* w, int nv, int B, int64_t N,
-                            double2* partial, int nblk, double2* out, cudaStream_t s, KernelTimer* tm);
+                            double2* partial, int nblk, double2* out, cudaStream_t s, KernelTimer* tm,
+                            double2* coef = nullptr, const double* act = nullptr);
 // w[b] += sum_i coef[b][i] V_i[b]  (coef device [B][nv])
 cudaError_t launch_multi_axpy(double2* w, const double2* V, int64_t vstride, const double2* coef, int nv,
                               int B, int64_t N, cudaStream_t s, KernelTimer* tm);
