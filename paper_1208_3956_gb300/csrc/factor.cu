@@ -143,9 +143,11 @@ __device__ void spike_solve(const Geom& g, const StripDev& st, const C* SinvS, C
     }
 }
 
-template <typename C, int NI>
-__global__ void __launch_bounds__(kBlockThreads) k_factor_chunk(Geom g, C* __restrict__ Sinv, C* __restrict__ GT,
-                                                                C* __restrict__ GB, int* __restrict__ status) {
+// MINB: CTAs to fit on an SM (0: as the registers come, two); see launch_factor_ni.
+template <typename C, int NI, int MINB>
+__global__ void __launch_bounds__(kBlockThreads, MINB) k_factor_chunk(Geom g, C* __restrict__ Sinv,
+                                                                      C* __restrict__ GT, C* __restrict__ GB,
+                                                                      int* __restrict__ status) {
     const StripDev st = g.strips[blockIdx.y];
     const int p = blockIdx.x;
     const int W = st.W;
@@ -399,15 +401,15 @@ struct SepStrip {
 // The separator system in three launches, each as wide as its dependencies allow.  One CTA per
 // strip ran all of it; with that, an uncoalesced read per spike entry, an FP64 division per
 // coupling and one product entry per thread, it took 33.5 ms of a 65 ms factorisation on the
-// 1023 x 1023 grid (64 strips) and 21 of 30 ms on 511 x 511 (32 strips); now 5.3 of 29.5 and
-// 2.2 of 9.6 ms, bound by the chain of block inversions of the longest group and of level 2.
+// 1023 x 1023 grid (64 strips) and 21 of 30 ms on 511 x 511 (32 strips); now 4.8 of 27.5 and
+// 2.2 of 9.0 ms, bound by the chain of block inversions of the longest group and of level 2.
 // k_factor_sep_group (group x strip): twisted LU of the group's separators, then the group
 // spikes, the response of the group to the level-2 separator above (right-hand side L_{q0} at
 // its first element) and below (U_{q1-1} at its last).
-template <typename C, int NI>
-__global__ void __launch_bounds__(kBlockThreads) k_factor_sep_group(Geom g, const C* __restrict__ GT,
-                                                                    const C* __restrict__ GB, SepPools<C> pl,
-                                                                    int* __restrict__ status) {
+template <typename C, int NI, int MINB>
+__global__ void __launch_bounds__(kBlockThreads, MINB) k_factor_sep_group(Geom g, const C* __restrict__ GT,
+                                                                          const C* __restrict__ GB, SepPools<C> pl,
+                                                                          int* __restrict__ status) {
     HELM_SEP_STRIP(g.G > 1)
     const int G = g.G, gi = blockIdx.x;
     const int q0 = g.gq0[gi], q1 = g.gq1[gi], n = q1 - q0, tq = (n - 1) / 2;
@@ -697,23 +699,34 @@ static cudaError_t launch_factor_ni(const Geom& g, int Wmax, void* const* pool, 
     };
     const size_t blk = (size_t)Wmax * Wmax * sizeof(C);
     const C *GT = (const C*)pool[1], *GB = (const C*)pool[2];
-    cudaError_t err = attr((const void*)k_factor_chunk<C, NI>, 3 * blk);
+    // A chunk's chain of inversions and products leaves most issue slots empty (barriers, shared
+    // memory), so a third CTA per SM helps once the grid has more than two for each: complex64
+    // 3 x 3 tiles fit in its 80 registers without spills.  Factor of 1023 x 1023 30.5 -> 27.5 ms,
+    // 511 x 511 9.6 -> 9.1; four CTAs (64 registers, spills) 27.9 and 9.35.  Smaller grids keep
+    // the registers (127 x 127: 2.75 ms against 2.79), and so does complex128, bound by the FP64
+    // pipe.
+    constexpr int kMinB = sizeof(C) == 8 && NI == 3 ? 3 : 0;
+    int dev = 0, nsm = 0;
+    cudaError_t err = cudaGetDevice(&dev);
     if (err != cudaSuccess) return err;
+    if ((err = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return err;
+    const auto chunk_fn = g.P * g.J > 2 * nsm ? k_factor_chunk<C, NI, kMinB> : k_factor_chunk<C, NI, 0>;
+    if ((err = attr((const void*)chunk_fn, 3 * blk)) != cudaSuccess) return err;
     {
         TimedLaunch t(tm, "factor_chunk", s);
-        k_factor_chunk<C, NI><<<dim3(g.P, g.J), kBlockThreads, 3 * blk, s>>>(g, (C*)pool[0], (C*)pool[1], (C*)pool[2],
-                                                                             status);
+        chunk_fn<<<dim3(g.P, g.J), kBlockThreads, 3 * blk, s>>>(g, (C*)pool[0], (C*)pool[1], (C*)pool[2], status);
     }
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
     if (g.P > 1) {
         SepPools<C> pl{(C*)pool[3], (C*)pool[4], (C*)pool[5], (C*)pool[6], (C*)pool[7], (C*)pool[8], (C*)pool[9],
                        g.G > 1 ? (C*)pool[11] : nullptr, g.G > 1 ? (C*)pool[12] : nullptr};
         const size_t smem = (g.G > 1 ? 4 : 3) * blk;
-        for (const void* fn : {(const void*)k_factor_sep_group<C, NI>, (const void*)k_factor_sep_l2<C, NI>,
+        const auto group_fn = g.G * g.J > 2 * nsm ? k_factor_sep_group<C, NI, kMinB> : k_factor_sep_group<C, NI, 0>;
+        for (const void* fn : {(const void*)group_fn, (const void*)k_factor_sep_l2<C, NI>,
                                (const void*)k_factor_sep_q<C, NI>})
             if ((err = attr(fn, smem)) != cudaSuccess) return err;
         TimedLaunch t(tm, "factor_sep", s);
-        k_factor_sep_group<C, NI><<<dim3(g.G, g.J), kBlockThreads, smem, s>>>(g, GT, GB, pl, status);
+        group_fn<<<dim3(g.G, g.J), kBlockThreads, smem, s>>>(g, GT, GB, pl, status);
         if (g.G > 1) {
             k_factor_sep_l2<C, NI><<<dim3(1, g.J), kBlockThreads, smem, s>>>(g, GT, GB, pl, status);
             k_factor_sep_q<C, NI><<<dim3(2 * g.G, g.J), kBlockThreads, smem, s>>>(g, GT, GB, pl, status);
