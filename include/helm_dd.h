@@ -127,6 +127,12 @@ int helm_dd_sep_groups(const helm_dd* h);
 /* P in use after helm_dd_factor (0 before). */
 int helm_dd_chunks(const helm_dd* h);
 
+/* Right-hand sides that a CTA of a 2-D strip solve carries when nrhs fields are
+ * applied together (0 before helm_dd_factor and on 3-D grids): 1 for one field,
+ * else 4 in complex64; in complex128 4 only once one-wide CTAs would take several
+ * rounds of the SMs. */
+int helm_dd_tile_width(const helm_dd* h, int nrhs);
+
 /* Most right-hand sides per internal panel of helm_dd_solve, helm_dd_solve_reduced
  * and helm_dd_gradient (the batching of many-source runs, not the paper's own
  * parameter): a call with more right-hand sides runs them panel after panel, so

@@ -126,7 +126,7 @@ struct helm_dd {
 
 namespace {
 
-constexpr int kMaxTiles = 4096;   // RHS tiles of one sweep launch (4 RHS per tile)
+constexpr int kMaxTiles = 4096;   // RHS tiles of one sweep launch (1 or 4 right-hand sides each)
 
 helm_status fail(helm_dd* h, helm_status s, const std::string& msg) {
     if (h) h->err = msg;
@@ -314,6 +314,8 @@ int work_stride(const helm_dd* h) { return (h->Wmax + 1) & ~1; }
 
 // one set per stream that runs strip solves (three for concurrent sweeps)
 int sweep_streams(const helm_dd* h) { return h->sweep == HELM_SWEEP_CONCURRENT ? 3 : 1; }
+// (concurrent sweeps of a single strip run as a double sweep)
+SweepShare sweep_share(const helm_dd* h) { return {h->nsm, h->J > 1 ? sweep_streams(h) : 1}; }
 size_t counter_set_bytes(const helm_dd* h) { return (size_t)kMaxTiles * (h->G + 1) * sizeof(int); }
 size_t counter_bytes(const helm_dd* h) { return counter_set_bytes(h) * sweep_streams(h); }
 
@@ -1040,7 +1042,7 @@ helm_status run_precond(helm_dd* h, const double2* in, double2* out, int B, cons
     CK(h, zero_acc2(h, bf.parts, B));
     auto strip_solve = [&](int j, const SweepStep& sp) -> cudaError_t {
         SweepWork wk{ybuf(j), bf.parts, bf.counters, h->d_status, ws, B, h->zrows,
-                     sp.prev >= 0 ? ybuf(sp.prev) : nullptr};
+                     sp.prev >= 0 ? ybuf(sp.prev) : nullptr, sweep_share(h)};
         const StripDev* pst = sp.prev >= 0 ? &h->strips[sp.prev] : nullptr;
         if (mixed)
             return launch_strip_solve<float2>(h->geom, j, h->strips[j], pst, sp, wk, h->d_pool, h->stream, &h->timer);
@@ -1209,7 +1211,7 @@ helm_status run_precond_concurrent(helm_dd* h, const double2* in, double2* out, 
     // set: 0 upward, 1 downward, 2 corrections; the transfer comes from set `pset`
     auto strip_solve = [&](int set, int j, const SweepStep& sp, int pset) -> cudaError_t {
         SweepWork wk{ybuf(set, j), parts[set], ctr[set], h->d_status, ws, B, h->zrows,
-                     sp.prev >= 0 ? ybuf(pset, sp.prev) : nullptr};
+                     sp.prev >= 0 ? ybuf(pset, sp.prev) : nullptr, sweep_share(h)};
         wk.pdl = false;   // a pre-launched successor would hold SMs the other streams need
         const StripDev* pst = sp.prev >= 0 ? &h->strips[sp.prev] : nullptr;
         if (mixed)
@@ -1636,7 +1638,7 @@ helm_status run_local_solves(helm_dd* h, const double2* F, double2* Ut, int B, c
     const int kOutBatch = 8;
     for (int j = 0; j < J; ++j) {
         const SweepStep sp = step_of(j);
-        SweepWork wk{ybuf(j), bf.parts, bf.counters, h->d_status, ws, B, h->zrows, nullptr};
+        SweepWork wk{ybuf(j), bf.parts, bf.counters, h->d_status, ws, B, h->zrows, nullptr, SweepShare{h->nsm, 1}};
         cudaError_t e = mixed ? launch_strip_solve<float2>(h->geom, j, h->strips[j], nullptr, sp, wk, h->d_pool,
                                                            h->stream, &h->timer)
                               : launch_strip_solve<double2>(h->geom, j, h->strips[j], nullptr, sp, wk, h->d_pool,
@@ -2099,6 +2101,14 @@ double helm_dd_precond_factor_bytes(const helm_dd* h) {
 void helm_dd_dims(const helm_dd* h, int64_t N[3]) {
     if (!h || !N) return;
     for (int a = 0; a < 3; ++a) N[a] = h->N[a];
+}
+
+int helm_dd_tile_width(const helm_dd* h, int nrhs) {
+    if (!h || !h->factored || h->dim != 2 || nrhs < 1) return 0;
+    int w = 4;
+    for (const auto& s : h->strips)
+        w = std::min(w, strip_solve_tile(h->geom, s, h->zrows, h->esize, nrhs, sweep_share(h)));
+    return w;
 }
 
 int helm_dd_strip_widths(const helm_dd* h, int* W, int cap) {

@@ -112,6 +112,11 @@ struct SweepStep {
 size_t sweep_parts_bytes(int P, int B, int Wmax, size_t esize);
 size_t sweep_parts_total_bytes(int P, int B, int Wmax, size_t esize);
 size_t sweep_parts2_bytes(int P, int B, int Wmax, size_t esize);   // the trailing level-2 accumulators
+// What a strip solve shares the GPU with: its SMs and how many streams run strip solves on them.
+struct SweepShare {
+    int nsm;
+    int streams;
+};
 struct SweepWork {
     void* ybuf;             // [B][Ny][Wmax] working precision (this strip's chain solution)
     void* parts;            // sweep_parts_total_bytes: parts, then level-2 contributions
@@ -121,6 +126,7 @@ struct SweepWork {
     int B;
     int zrows;              // longest chain of one CTA (chunk rows, group size, G-1)
     const void* pybuf;      // the previous strip solve's chain solution (when SweepStep::prev >= 0)
+    SweepShare share;
     // launch with programmatic stream serialisation (the next strip solve's CTAs stage their
     // blocks while this one finishes); off where strip solves of several streams share the SMs
     bool pdl = true;
@@ -145,6 +151,8 @@ cudaError_t launch_outputs(const OutArgs& O, void* const* pool, cudaStream_t s, 
 // Whether one strip solve of st (a ring of at least four W x W blocks in shared memory)
 // fits on an SM with elements of esize bytes.
 bool strip_solve_fits(const StripDev& st, int zrows, size_t esize);
+// Right-hand sides per tile of a strip solve of st with B right-hand sides (4 or 1).
+int strip_solve_tile(const Geom& g, const StripDev& st, int zrows, size_t esize, int B, const SweepShare& share);
 
 template <typename C>
 // pst: the strip of the previous solve whose transfer enters this one (step.prev >= 0), host copy

@@ -253,7 +253,7 @@ __device__ __forceinline__ void dual_rows_r(const C (&sd)[NJ], const C (&su)[NJ]
     }
 }
 
-// Compute warps of a tile of several right-hand sides (BT = 4, complex64).  Half of the warps run
+// Compute warps of a tile of several right-hand sides (BT = 4).  Half of the warps run
 // the down chain of a step, half the up chain (a step's products are then one instruction
 // stream per chain, side by side), each half as (pair of right-hand sides) x (16 rows).  A lane
 // owns one row and half of the columns: 16-byte reads of the block's rows (conflict-free with
@@ -718,6 +718,9 @@ __global__ void __launch_bounds__(BT == 1 ? 288 : chunk_threads(4 * NJ, BT)) k_s
     const bool upw = kPanel && w >= 2 * nrb;                    // panel: a warp of the up chain
     const int bp = kPanel ? (w / nrb) & 1 : 0;                  // panel: pair of right-hand sides
     const int ob = 2 * bp + g;                                  // panel: the right-hand side this lane finishes
+    // panel: the warp's pair has a right-hand side (a ragged tile's absent pair multiplies nothing; its
+    // products cost a complex128 tile of 1 or 2 as much FP64 pipe as the present ones)
+    const bool pairon = compute && 2 * bp < nb;
     const bool rowok = compute && row < W;
     const bool own = kPanel && rowok && ob < nb;
     const int rc = imin(row, W - 1);
@@ -822,7 +825,7 @@ __global__ void __launch_bounds__(BT == 1 ? 288 : chunk_threads(4 * NJ, BT)) k_s
                      C ckd, C cku, bool wvd, bool wvu, R az, R sv, R ez, R fc, bool pd = false, bool pu = false,
                      const C* pbase = nullptr, R ps = (R)1) -> bool {
         if constexpr (kPanel) {   // each half of the warps its chain
-            if (compute && (upw ? U : D)) {
+            if (pairon && (upw ? U : D)) {
                 C* z = (upw ? zu : zd) + ob * W;
                 const C* zn = (upw ? znu : znd) + ob * W;
                 const C ck = upw ? cku : ckd;
@@ -914,7 +917,7 @@ __global__ void __launch_bounds__(BT == 1 ? 288 : chunk_threads(4 * NJ, BT)) k_s
         step2(St, vin_d, St, vin_d);
         const C cd = cpl(t), cu = cpl(t + 1);
         if constexpr (kPanel) {
-            if (compute && !upw) {
+            if (pairon && !upw) {
                 const C v = prod(St, vin_d);
                 if (own) {
                     zr(t)[ob * W + row] = v;
@@ -988,7 +991,7 @@ __global__ void __launch_bounds__(BT == 1 ? 288 : chunk_threads(4 * NJ, BT)) k_s
         consume_ab(has_below, has_above, SA, SB);
         step2(has_below ? SA : SB, has_below ? pv_u : pv_d, has_above ? SB : SA, has_above ? pv_d : pv_u);
         if constexpr (kPanel) {
-            if (compute) {
+            if (pairon) {
                 const bool on_ = upw ? has_above : has_below;
                 const C v = on_ ? prod(upw ? SB : SA, upw ? pv_d : pv_u) : CT<C>::zero();
                 if (own) {
@@ -1029,7 +1032,7 @@ __global__ void __launch_bounds__(BT == 1 ? 288 : chunk_threads(4 * NJ, BT)) k_s
             if (!a && !b) return;
             const C *SA, *SB;
             consume_ab(a, b, SA, SB);
-            if (compute && (upw ? b : a)) {
+            if (pairon && (upw ? b : a)) {
                 const C v = prod(upw ? SB : SA, upw ? vin_u : vin_d);
                 if (own) catomic_add(acc2 + a2idx(ob, r) + row, v);
             }
@@ -1127,7 +1130,7 @@ __global__ void __launch_bounds__(BT == 1 ? 288 : chunk_threads(4 * NJ, BT)) k_s
             step2(he ? Se : Sf, he ? vin_d : vin_u, hf ? Sf : Se, hf ? vin_u : vin_d);
             if constexpr (kPanel) {
                 const bool on_ = upw ? hf : he;
-                const C v = (compute && on_) ? prod(upw ? Sf : Se, upw ? vin_u : vin_d) : CT<C>::zero();
+                const C v = (pairon && on_) ? prod(upw ? Sf : Se, upw ? vin_u : vin_d) : CT<C>::zero();
                 if (upw && own) vout_u[ob * 64 + row] = v;   // to the lane that sums both terms
                 __syncthreads();
                 if (!upw && own) {
@@ -1625,15 +1628,33 @@ static SweepArgs make_args(const Geom& g, const StripDev& st, const SweepStep& s
     return A;
 }
 
-// Largest ring (and RHS tile) that fits the shared-memory budget.
+// Right-hand sides of a tile (a CTA): 4 or 1, before the shared-memory limit.  Complex64: 4 whenever
+// there are several.  Complex128 is bound by the FP64 pipe of the SMs that run a strip solve.  While
+// its one-wide CTAs leave SMs idle or take a few rounds of them, separate CTAs spread the work (447 x
+// 383 grid, one P with 2 / 4 / 8 right-hand sides: 9.3 / 15.4 / 27.0 ms, in 4-wide tiles 20.3 / 24.0 /
+// 29.4); once the SMs are full anyway, a 4-wide tile does a third more per SM (four right-hand sides
+// hide each other's latencies and stream the blocks once): 32 / 64 / 128 right-hand sides 95 / 187 /
+// 370 ms one-wide, 88 / 169 / 335 in tiles.  The sides meet at 4 to 9 rounds of one-wide CTAs where a
+// solve has the GPU to itself (511 x 511, 16: 6.6 rounds, 66.7 and 62.0 ms; 127 x 127, 32: 5.7
+// rounds, 9.2 and 9.8 ms): the line is at 8.  Strip solves of three streams fill each other's gaps and
+// meet at 4 to 5 (255 x 255 concurrent, 5 / 6 / 8: 4.0 / 4.9 / 6.5 rounds, 6.7 / 8.0 / 10.7 ms one-wide,
+// 7.4 / 7.9 / 9.4 in tiles): the line is at 4.5.
 template <typename C>
-static bool plan(const StripDev& st, int zrows, int B, int& Bt, int& ring, size_t& smem) {
+static int tile_width(int B, int ctas, const SweepShare& sh) {
+    if (B == 1) return 1;
+    if (sizeof(C) == sizeof(float2)) return 4;
+    const double rounds = (double)B * ctas * sh.streams / imax(sh.nsm, 1);
+    return rounds > (sh.streams > 1 ? 4.5 : 8.0) ? 4 : 1;
+}
+// CTAs of a tile: one per chunk, with separator groups one more for level 2
+static int tile_ctas(int P, int G) { return P + (G > 1 ? 1 : 0); }
+
+// Largest ring (and RHS tile, at most Bt wide) that fits the shared-memory budget.
+template <typename C>
+static bool plan(const StripDev& st, int zrows, int& Bt, int& ring, size_t& smem) {
     const size_t budget = 220 * 1024;
     const uint32_t slot = (uint32_t)(st.bs * sizeof(C));
-    // tiles of 4 right-hand sides in complex64, or 1.  Complex128 is bound by the FP64 pipe of the
-    // SMs that run a strip solve, so its right-hand sides go to separate CTAs (511 x 511 grid, two
-    // right-hand sides: 18.9 ms for one P in one 4-wide tile, 11.5 ms in two tiles)
-    for (Bt = (B > 1 && sizeof(C) == sizeof(float2) ? 4 : 1); Bt >= 1; Bt -= 3) {
+    for (; Bt >= 1; Bt -= 3) {   // tiles of 4 right-hand sides, or 1
         for (ring = kMaxRing; ring >= 4; --ring) {
             smem = sweep_smem(ring, slot, zrows, Bt, st.W, (int)sizeof(C)).total;
             if (smem <= budget) return true;
@@ -1642,11 +1663,19 @@ static bool plan(const StripDev& st, int zrows, int B, int& Bt, int& ring, size_
     return false;
 }
 
-bool strip_solve_fits(const StripDev& st, int zrows, size_t esize) {
-    int Bt, ring;
+template <typename C>
+static int planned_tile(const StripDev& st, int zrows, int Bt) {
+    int ring;
     size_t smem;
-    return esize == sizeof(float2) ? plan<float2>(st, zrows, 1, Bt, ring, smem)
-                                   : plan<double2>(st, zrows, 1, Bt, ring, smem);
+    return plan<C>(st, zrows, Bt, ring, smem) ? Bt : 0;
+}
+bool strip_solve_fits(const StripDev& st, int zrows, size_t esize) {
+    return (esize == sizeof(float2) ? planned_tile<float2>(st, zrows, 1) : planned_tile<double2>(st, zrows, 1)) > 0;
+}
+int strip_solve_tile(const Geom& g, const StripDev& st, int zrows, size_t esize, int B, const SweepShare& sh) {
+    const int ctas = tile_ctas(g.P, g.G);
+    return esize == sizeof(float2) ? planned_tile<float2>(st, zrows, tile_width<float2>(B, ctas, sh))
+                                   : planned_tile<double2>(st, zrows, tile_width<double2>(B, ctas, sh));
 }
 
 // Shared-memory limit of every strip-solve instantiation (this also loads the module).
@@ -1657,12 +1686,9 @@ static cudaError_t chunk_kernel_attrs() {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
     };
     for (auto fn : {k_sweep_chunk<C, 8, 1>, k_sweep_chunk<C, 10, 1>, k_sweep_chunk<C, 12, 1>, k_sweep_chunk<C, 14, 1>,
-                    k_sweep_chunk<C, 16, 1>})
+                    k_sweep_chunk<C, 16, 1>, k_sweep_chunk<C, 8, 4>, k_sweep_chunk<C, 10, 4>, k_sweep_chunk<C, 12, 4>,
+                    k_sweep_chunk<C, 14, 4>, k_sweep_chunk<C, 16, 4>})
         set(fn);
-    if constexpr (sizeof(C) == sizeof(float2))
-        for (auto fn : {k_sweep_chunk<C, 8, 4>, k_sweep_chunk<C, 10, 4>, k_sweep_chunk<C, 12, 4>,
-                        k_sweep_chunk<C, 14, 4>, k_sweep_chunk<C, 16, 4>})
-            set(fn);
     return e;
 }
 
@@ -1680,9 +1706,10 @@ template <typename C>
 cudaError_t launch_strip_solve(const Geom& g, int j, const StripDev& st, const StripDev* pst,
                                const SweepStep& step, const SweepWork& wk, void* const* pool, cudaStream_t s,
                                KernelTimer* tm) {
-    int Bt, ring;
+    const int ctas = tile_ctas(g.P, g.G);
+    int Bt = tile_width<C>(wk.B, ctas, wk.share), ring;
     size_t smem;
-    if (!plan<C>(st, wk.zrows, wk.B, Bt, ring, smem)) return cudaErrorInvalidConfiguration;
+    if (!plan<C>(st, wk.zrows, Bt, ring, smem)) return cudaErrorInvalidConfiguration;
     static bool attr_set = false;
     if (!attr_set) {
         cudaError_t e = chunk_kernel_attrs<C>();
@@ -1712,8 +1739,7 @@ cudaError_t launch_strip_solve(const Geom& g, int j, const StripDev& st, const S
     cudaError_t err;
     {
         void (*kfn)(SweepArgs) = nullptr;
-        constexpr int kBt = sizeof(C) == sizeof(float2) ? 4 : 1;
-#define HELM_CHUNK_FN(NJ) kfn = Bt == 1 ? k_sweep_chunk<C, NJ, 1> : k_sweep_chunk<C, NJ, kBt>
+#define HELM_CHUNK_FN(NJ) kfn = Bt == 1 ? k_sweep_chunk<C, NJ, 1> : k_sweep_chunk<C, NJ, 4>
         switch (st.nj) {
             case 8: HELM_CHUNK_FN(8); break;
             case 10: HELM_CHUNK_FN(10); break;
@@ -1722,8 +1748,8 @@ cudaError_t launch_strip_solve(const Geom& g, int j, const StripDev& st, const S
             default: HELM_CHUNK_FN(16); break;
         }
 #undef HELM_CHUNK_FN
-        // compute warps + the producer warp; with separator groups one more CTA for level 2
-        const cudaLaunchConfig_t cfg = config(dim3(g.P + (g.G > 1 ? 1 : 0), ntile), chunk_threads(st.W, Bt), smem);
+        // compute warps + the producer warp
+        const cudaLaunchConfig_t cfg = config(dim3(ctas, ntile), chunk_threads(st.W, Bt), smem);
         TimedLaunch t(tm, "sweep_chunk", s);
         err = cudaLaunchKernelEx(&cfg, kfn, A);
     }

@@ -57,6 +57,7 @@ def load() -> ctypes.CDLL:
         "helm_dd_set_sep_groups": (I, [P, I]),
         "helm_dd_sep_groups": (I, [P]),
         "helm_dd_chunks": (I, [P]),
+        "helm_dd_tile_width": (I, [P, I]),
         "helm_dd_set_panel": (I, [P, I]),
         "helm_dd_set_transmission": (I, [P, I]),
         "helm_dd_set_sweep": (I, [P, I]),
@@ -207,6 +208,10 @@ class HelmDD:
     def chunks(self) -> int:
         """The chunk count P in use after factor (0 before)."""
         return int(self.lib.helm_dd_chunks(self._h))
+
+    def tile_width(self, nrhs: int) -> int:
+        """Right-hand sides per CTA of a 2-D strip solve with nrhs fields (0 before factor, and in 3-D)."""
+        return int(self.lib.helm_dd_tile_width(self._h, int(nrhs)))
 
     def precond_factor_bytes(self) -> float:
         return float(self.lib.helm_dd_precond_factor_bytes(self._h))
