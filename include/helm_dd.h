@@ -109,7 +109,8 @@ helm_status helm_dd_set_pml_speed(helm_dd* h, double c_ref);
  * block-tridiagonal factorisation (1 = plain sequential block LU).  0 selects the
  * built-in choice: about 0.93 N_y^(2/3), lowered when a panel of more than 4
  * right-hand sides is set before helm_dd_factor (helm_dd_set_panel) so that the
- * panel's tiles of 4 fit one wave of the SMs.  Must be called before helm_dd_factor. */
+ * panel's tiles of 4 fit one wave of the SMs (complex64), or its CTAs of one right-hand
+ * side each fill whole rounds of them (complex128).  Must be called before helm_dd_factor. */
 helm_status helm_dd_set_chunks(helm_dd* h, int P);
 
 /* Number of groups G the P-1 separator rows of every strip are cut into (a

@@ -249,6 +249,16 @@ cd strip_alpha_at(const helm_dd* h, const StripDev& s, int x2) {
     return axis_alpha_at(po, (int)h->N[0], g2);
 }
 
+// Whether a strip solve on P chunks has its longest chunk in shared memory for every strip.
+bool chunks_fit(const helm_dd* h, int P) {
+    const int Ny = (int)h->N[1], rows = (Ny - (P - 1) + P - 1) / P;
+    for (StripDev s : h->strips) {
+        s.bs = (int64_t)s.W * (4 * sweep_nj(s.W) + 2);
+        if (!strip_solve_fits(s, rows, h->esize)) return false;
+    }
+    return true;
+}
+
 void chunk_layout(helm_dd* h) {
     const int Ny = (int)h->N[1];
     // built-in: a strip solve takes about Ny/P (chunk) + P/G (separator group) + G
@@ -256,14 +266,29 @@ void chunk_layout(helm_dd* h) {
     // factor 0.93 (fewer, longer chunks) is the measured optimum on a 1055-row grid,
     // where the chunk steps are slightly cheaper than the separator steps.
     int P = h->P_req > 0 ? h->P_req : std::max(1, (int)lround(0.93 * pow((double)Ny, 2.0 / 3.0)));
-    // A panel of B > 4 right-hand sides (set before the factorisation) runs each strip
-    // solve as ceil(B/4) tiles of P+1 CTAs (one SM each).  Once the tiles exceed one wave
-    // of the SMs they run one after another, so the built-in count drops to the P whose
-    // tiles all fit one wave, but not below a sixth of it (longer chunk chains).  On 1055
-    // rows this halves the time per right-hand side at B = 32 (P = 18 against 96).
+    // A panel of B > 4 right-hand sides (set before the factorisation) runs each strip solve as
+    // tiles of P+1 CTAs (one SM each), and the built-in count drops for it (longer chunk chains),
+    // to a sixth at most and not below what a strip solve's shared memory holds.
+    // Tiles of 4 (complex64; complex128 concurrent sweeps, whose panels run in such tiles): once
+    // the tiles exceed one wave of the SMs they run one after another, so P is the one whose tiles
+    // all fit one wave.  Complex64 on 1055 rows: half the time per right-hand side at B = 32 (P = 18
+    // against 96).
+    // Complex128, one right-hand side to a CTA: P fills the fewest whole rounds of the SMs, since a
+    // round begun costs nearly a full one, with P not below what one round holds of 8 right-hand
+    // sides (or of tiles of 4, where that is less): fewer and longer chunks gain up to 15 % more on
+    // 147 rows and nothing on 735 and 1055.  P f on 415 rows with 8 / 16 / 24 right-hand sides:
+    // 11.4 / 19.1 / 27.5 ms (P = 18 in 1, 2 and 3 rounds) against 13.5 / 22.0 / 28.6 at one wave of
+    // tiles of 4 (P = 52, 37, 24).
     if (h->P_req == 0 && h->panel > 4 && h->nsm > 0) {
-        const int tiles = (h->panel + 3) / 4;
-        P = std::min(P, std::max(h->nsm / tiles - 1, (P + 5) / 6));
+        const int tiles = (h->panel - 1) / 4 + 1, least = (P + 5) / 6, most = P;
+        if (h->esize == sizeof(float2) || h->sweep == HELM_SWEEP_CONCURRENT) {
+            P = std::min(P, std::max(h->nsm / tiles - 1, least));
+        } else {
+            const int low = std::max(h->nsm / std::max(tiles, 8) - 1, least);
+            const int64_t rounds = ((int64_t)(low + 1) * h->panel + h->nsm - 1) / h->nsm;
+            P = (int)std::min<int64_t>(P, rounds * h->nsm / h->panel - 1);
+        }
+        while (h->dim == 2 && P < most && !chunks_fit(h, P)) ++P;
     }
     // concurrent sweeps run three strip solves side by side (one CTA per chunk and SM, and
     // one for the level-2 system)
