@@ -417,6 +417,7 @@ helm_status ensure_device(helm_dd* h) {
     CK(h, noalloc_scratch(&h->noalloc_base));
     CK(h, preload_sweep_kernels());
     CK(h, preload_slab_kernels());
+    CK(h, preload_tc_kernels());
     CK(h, preload_field_kernels());
     const int64_t nint = (int64_t)h->c.size();
     CK(h, cudaMalloc(&h->d_c, nint * sizeof(double)));

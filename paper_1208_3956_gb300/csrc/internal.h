@@ -209,11 +209,13 @@ template <typename C>
 cudaError_t launch_slab_out(const Geom& g, const StripDev& st, int dir, const void* ybuf, int ld, double2* dst,
                             const double2* base, int B, cudaStream_t s, KernelTimer* tm);
 
-// Load the modules of each file's kernels onto the current device (lazy module
-// loading would otherwise load them, and take their memory, at the first launch
-// inside some later call).
+// Load each file's kernels onto the current device (lazy loading would otherwise load them,
+// and take their memory, at the first launch inside some later call) and set the
+// shared-memory limits of those that need more than 48 KB; once per handle, at its first
+// device use.
 cudaError_t preload_sweep_kernels();
 cudaError_t preload_slab_kernels();
+cudaError_t preload_tc_kernels();
 cudaError_t preload_field_kernels();
 
 // ---- field.cu: FP64 grid kernels

@@ -40,6 +40,7 @@ constexpr uint32_t kBarPolls = 1u << 20;   // polls of a grid barrier before it 
 constexpr int kGjThreads = 256;
 constexpr int kGjRowsPerThread = 8;        // n <= kGjThreads * kGjRowsPerThread
 constexpr int kGjMaxCols = 64;             // columns owned by one CTA
+constexpr size_t kGjCacheMax = 200 * 1024; // the owned columns in shared memory, at most
 
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
     unsigned v;
@@ -705,16 +706,9 @@ cudaError_t launch_slab_factor(const Geom& g, const StripDev& st, void* pool, co
     const int nb = imin(nsm, n);
     if ((n + nb - 1) / nb > kGjMaxCols) return cudaErrorInvalidConfiguration;
     // the owned columns stay in shared memory when they fit
-    const size_t kCacheMax = 200 * 1024;
     const size_t cache = (size_t)((n + nb - 1) / nb) * n * sizeof(C);
-    int cached = cache <= kCacheMax ? 1 : 0;
+    int cached = cache <= kGjCacheMax ? 1 : 0;
     size_t dsmem = cached ? cache : 0;
-    static bool attr_set = false;
-    if (!attr_set) {
-        e = cudaFuncSetAttribute(k_gj_invert<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCacheMax);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_gj_invert<C>, kGjThreads, dsmem);
     if (e != cudaSuccess) return e;
     if (occ < 1) return cudaErrorInvalidConfiguration;
@@ -809,9 +803,10 @@ static cudaError_t sm_count(int& nsm) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     return e;
 }
+// Shared-memory limits of every variant on the current device (this also loads them).
 template <typename C>
-static cudaError_t slab_sweep_attrs() {
-    cudaError_t e = cudaSuccess;
+static cudaError_t slab_kernel_attrs() {
+    cudaError_t e = cudaFuncSetAttribute(k_gj_invert<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGjCacheMax);
     auto set = [&](const void* fn) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     };
@@ -855,12 +850,6 @@ cudaError_t launch_slab_solve(const Geom& g, const StripDev& st, const StripDev*
     int nsm = 0;
     e = sm_count(nsm);
     if (e != cudaSuccess) return e;
-    static bool attr_set = false;
-    if (!attr_set) {
-        e = slab_sweep_attrs<C>();
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
     if (n > 128 * kMaxRowTiles) return cudaErrorInvalidValue;
     const SlabGrid gr = slab_grid(n, nsm);
     for (int b0 = 0; b0 < B;) {
@@ -909,14 +898,13 @@ cudaError_t launch_slab_out(const Geom& g, const StripDev& st, int dir, const vo
     return cudaGetLastError();
 }
 
-// Loads this file's module onto the current device (the strip-solve kernels of a
-// preconditioner application).
+// Loads this file's kernels onto the current device and sets their shared-memory limits there.
 cudaError_t preload_slab_kernels() {
     cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, k_slab_rhs<float2>);
+    cudaError_t e = slab_kernel_attrs<float2>();
+    if (e == cudaSuccess) e = slab_kernel_attrs<double2>();
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_rhs<float2>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_rhs<double2>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_sweep<float2, 1>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_sweep<double2, 1>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_out<float2>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_out<double2>);
     return e;

@@ -574,6 +574,14 @@ __global__ void __launch_bounds__(256) k_tc_store(const __grid_constant__ TcArgs
     S.X[slab_at(n, r, c)] = (pc < n && q >= 0 && q < n) ? S.M[(int64_t)pc * S.ldm + q] : make_float2(0.f, 0.f);
 }
 
+// Loads the update kernels onto the current device and sets their shared-memory limit there.
+cudaError_t preload_tc_kernels() {
+    cudaError_t e = cudaFuncSetAttribute(k_tc_update<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcUpdSmem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_tc_update<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcUpdSmem);
+    return e;
+}
+
 size_t slab_factor_tc_scratch(int nmax, int ns) {
     const int npad = (nmax + kTcRows - 1) / kTcRows * kTcRows;
     const size_t ldm = (size_t)((nmax + 3) & ~3);
@@ -585,17 +593,9 @@ size_t slab_factor_tc_scratch(int nmax, int ns) {
 cudaError_t launch_slab_factor_tc(const Geom& g, const StripDev* strips, int ns, void* pool, void* scratch,
                                   int* status, cudaStream_t s, KernelTimer* tm) {
     if (ns < 1 || ns > kTcMaxStrips) return cudaErrorInvalidValue;
-    static bool attr_set = false;
     int nmax = 0;
     for (int i = 0; i < ns; ++i) nmax = imax(nmax, strips[i].W * g.Nz);
     if (nmax > kTcPanelSpan * kTcPanelRows) return cudaErrorInvalidValue;   // the block limit
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_tc_update<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcUpdSmem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_tc_update<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcUpdSmem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
     TcArgs A{};
     A.status = status;
     auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };

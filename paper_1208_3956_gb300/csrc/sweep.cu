@@ -1710,12 +1710,6 @@ cudaError_t launch_strip_solve(const Geom& g, int j, const StripDev& st, const S
     int Bt = tile_width<C>(wk.B, ctas, wk.share), ring;
     size_t smem;
     if (!plan<C>(st, wk.zrows, Bt, ring, smem)) return cudaErrorInvalidConfiguration;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = chunk_kernel_attrs<C>();
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
     SweepArgs A = make_args<C>(g, st, step, wk, pool, Bt, ring);
     if (pst && step.prev >= 0) {
         A.has_prev = 1;
