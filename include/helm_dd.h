@@ -190,7 +190,9 @@ helm_status helm_dd_set_transmission(helm_dd* h, helm_transmission t);
  * HELM_ETIMEOUT.  HELM_EINVAL when a 3-D block exceeds 4096 unknowns in complex64
  * or 2048 in complex128 (use more strips).  Factor memory: N_y n^2 complex entries
  * per strip (8 or 16 bytes), rows rounded up to 64, and a few MB for the strip
- * solve's vectors and partial sums. */
+ * solve's vectors and partial sums; while it runs, complex64 takes two more blocks for
+ * each strip it factors side by side (up to 8 strips, fewer when memory is short),
+ * complex128 two in all. */
 helm_status helm_dd_factor(helm_dd* h);
 
 /* out = P in for nrhs right-hand sides (Section 2.1, Eqs. solve_upward and

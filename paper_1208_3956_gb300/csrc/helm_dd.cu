@@ -696,45 +696,49 @@ helm_status factor_slabs(helm_dd* h) {
     CK(h, cudaMemcpyAsync(h->d_strips, h->strips.data(), h->strips.size() * sizeof(StripDev),
                           cudaMemcpyHostToDevice, h->stream));
     CK(h, cudaMemsetAsync(h->d_status, 0, sizeof(int), h->stream));
-    // scratch of the block inversions
-    const size_t es = h->esize;
-    const size_t mbytes = (size_t)ldmax * nmax * es, multb = (size_t)nmax * ldmax * es;
-    const size_t ibytes = (size_t)(3 * nmax + 2) * sizeof(int);
+    // the block inversions and their scratch, freed at the end
     void* scratch = nullptr;
-    CK(h, cudaMalloc(&scratch, mbytes + multb + ibytes));
-    SlabScratch sc{};
-    sc.M = scratch;
-    sc.mult = (char*)scratch + mbytes;
-    sc.ldm = ldmax;
-    sc.perm = (int*)((char*)scratch + mbytes + multb);
-    sc.pinv = sc.perm + nmax;
-    sc.pivrow = sc.pinv + nmax;
-    sc.bar = (unsigned*)(sc.pivrow + nmax);
     cudaError_t e = cudaSuccess;
     if (h->prec == HELM_PREC_MIXED) {
-        // complex64: blocked Gauss-Jordan with tensor-core updates, up to 8 strips side by side
-        const int ns_max = 8;
-        void* tcs = nullptr;
-        const size_t tcb = slab_factor_tc_scratch(nmax, std::min<int>(ns_max, (int)h->strips.size()));
-        e = cudaMalloc(&tcs, tcb);
+        // complex64: blocked Gauss-Jordan with tensor-core updates, up to 8 strips (16 chains of n^2
+        // entries each) side by side, half as many while the device memory left does not hold them
+        int ns_max = std::min<int>(8, (int)h->strips.size());
+        while ((e = cudaMalloc(&scratch, slab_factor_tc_scratch(nmax, ns_max))) == cudaErrorMemoryAllocation &&
+               ns_max > 1) {
+            cudaGetLastError();
+            ns_max = (ns_max + 1) / 2;
+        }
         for (size_t j0 = 0; j0 < h->strips.size() && e == cudaSuccess; j0 += ns_max) {
             const int ns = (int)std::min<size_t>(ns_max, h->strips.size() - j0);
-            e = launch_slab_factor_tc(h->geom, h->strips.data() + j0, ns, h->d_pool[0], tcs, h->d_status, h->stream,
-                                      &h->timer);
+            e = launch_slab_factor_tc(h->geom, h->strips.data() + j0, ns, h->d_pool[0], scratch, h->d_status,
+                                      h->stream, &h->timer);
         }
-        if (tcs) {
-            cudaError_t e2 = cudaStreamSynchronize(h->stream);
-            if (e == cudaSuccess) e = e2;
-            cudaFree(tcs);
-        }
+    } else {
+        // complex128: one block at a time
+        const size_t mbytes = (size_t)ldmax * nmax * h->esize;
+        SlabScratch sc{};
+        e = cudaMalloc(&scratch, 2 * mbytes + (size_t)(3 * nmax + 2) * sizeof(int));
+        sc.M = scratch;
+        sc.mult = (char*)scratch + mbytes;
+        sc.ldm = ldmax;
+        sc.perm = (int*)((char*)scratch + 2 * mbytes);
+        sc.pinv = sc.perm + nmax;
+        sc.pivrow = sc.pinv + nmax;
+        sc.bar = (unsigned*)(sc.pivrow + nmax);
+        for (size_t jj = 0; jj < h->strips.size() && e == cudaSuccess; ++jj)
+            e = launch_slab_factor<double2>(h->geom, h->strips[jj], h->d_pool[0], sc, h->d_status, h->stream,
+                                            &h->timer);
     }
-    for (size_t jj = 0; jj < h->strips.size() && e == cudaSuccess && h->prec != HELM_PREC_MIXED; ++jj)
-        e = launch_slab_factor<double2>(h->geom, h->strips[jj], h->d_pool[0], sc, h->d_status, h->stream, &h->timer);
+    const cudaError_t idle = cudaStreamSynchronize(h->stream);   // no launch of a failed sequence outlives the scratch
+    if (e == cudaSuccess) e = idle;
     int st = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&st, h->d_status, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     cudaFree(scratch);
-    if (e != cudaSuccess) return fail_cuda(h, "3-D strip factor kernels", e);
+    if (e != cudaSuccess) {
+        cudaGetLastError();   // a refused allocation is not the next launch's error
+        return fail_cuda(h, "3-D strip factor kernels", e);
+    }
     if (st == 7) {
         cudaMemsetAsync(h->d_status, 0, sizeof(int), h->stream);
         return fail(h, HELM_ETIMEOUT, "a bounded device wait in the 3-D strip factorisation gave up");
