@@ -268,8 +268,8 @@ __global__ void k_slab_rhs(Geom g, StripDev st, SweepStep sp, StripDev pst, cons
 //   sum:     the CTA's own `epc` entries of its row tile: y = sum over q of P (plus y_k on the
 //            way out), stored to Y, and the next step's z = r - C y on them, counter vec[m]
 //            raised.
-// A CTA's sums wait for the nq CTAs of its row tile only, and its copy of z for the two or three
-// row tiles that hold its columns.  Z and P are double buffered by the step's parity: a CTA
+// A CTA's sums wait for the nq CTAs of its row tile only, and its copy of z for the row tiles that
+// hold its kc columns (two or three at 1800 unknowns, up to nine at 4000).  Z and P are double buffered by the step's parity: a CTA
 // enters product s+2 after the products s+1 of its row tile, each of which followed its
 // CTA's sums of step s; and it writes z of step s+2 after all of its row tile's products
 // s+1, which together waited for every CTA's z of step s+1 and so for every product s.
