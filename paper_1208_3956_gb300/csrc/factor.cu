@@ -234,7 +234,7 @@ struct SepPools {
     C* Rinv;   // per separator slot, sweep layout
     C* E;
     C* F;
-    C* GT2;    // group spikes, row-major W x W
+    C* GT2;    // group spikes, W rows of spld(W)
     C* GB2;
     C* P2L;    // level-2 right-hand-side products Rinv2 L, Rinv2 U (sweep layout)
     C* P2U;
@@ -688,7 +688,8 @@ __global__ void k_factor_xfer(Geom g, const C* __restrict__ GT, const C* __restr
 }
 
 size_t factor_smem_bytes(int Wmax, size_t esize, int nbuf) {
-    return (size_t)nbuf * Wmax * Wmax * esize + (size_t)3 * Wmax * esize + (size_t)((Wmax + 3) & ~3) * 4 + 16;
+    const size_t fixed = 8 * 64 * esize + 64 * sizeof(int) + 64 * sizeof(double2);   // InvScratch, dv, dr; sx
+    return (size_t)nbuf * Wmax * Wmax * esize + fixed;
 }
 
 template <typename C, int NI>

@@ -99,12 +99,10 @@ struct helm_dd {
                         nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     int* d_status = nullptr;
     // 3-D strips: s_x s_z per block entry (working precision) and its per-strip offsets,
-    // the offset of s_z in d_ct, the y-couplings -alpha_y(y_{k-1/2})/h^2 and the row
-    // stride of the strip right-hand-side / solution buffers
+    // the offset of s_z in d_ct and the row stride of the strip right-hand-side / solution buffers
     void* d_slab_sxz = nullptr;
     std::vector<int64_t> slab_sxz_off;
     int64_t ct_sz = 0;
-    std::vector<double2> slab_cy;
     int slab_ld = 0;
     void* d_slab_scratch = nullptr;   // step vectors and partial sums of the 3-D strip solve
     size_t esize = 16;
@@ -665,7 +663,7 @@ helm_status factor_slabs(helm_dd* h) {
     for (auto& p : h->d_pool) { if (p) cudaFree(p); p = nullptr; }
     h->factored = false;
     CK(h, cudaMalloc(&h->d_pool[0], (size_t)fac * h->esize));
-    // s_x(c) s_z(z) per block entry, and the y-couplings
+    // s_x(c) s_z(z) per block entry
     std::vector<cd> sxz;
     h->slab_sxz_off.assign(h->strips.size(), 0);
     for (size_t jj = 0; jj < h->strips.size(); ++jj) {
@@ -674,9 +672,6 @@ helm_status factor_slabs(helm_dd* h) {
         for (int z = 0; z < Nz; ++z)
             for (int c = 0; c < s.W; ++c) sxz.push_back(1.0 / (strip_alpha_at(h, s, 2 * c) * h->gz_int[z]));
     }
-    const double ih2 = 1.0 / (h->h * h->h);
-    h->slab_cy.assign(Ny + 1, make_double2(0.0, 0.0));
-    for (int k = 0; k <= Ny; ++k) h->slab_cy[k] = to_d2h(-h->gy_half[k] * ih2);
     if (h->d_slab_sxz) cudaFree(h->d_slab_sxz);
     h->d_slab_sxz = nullptr;
     CK(h, cudaMalloc(&h->d_slab_sxz, sxz.size() * h->esize));
@@ -726,7 +721,7 @@ helm_status factor_slabs(helm_dd* h) {
         sc.pivrow = sc.pinv + nmax;
         sc.bar = (unsigned*)(sc.pivrow + nmax);
         for (size_t jj = 0; jj < h->strips.size() && e == cudaSuccess; ++jj)
-            e = launch_slab_factor<double2>(h->geom, h->strips[jj], h->d_pool[0], sc, h->d_status, h->stream,
+            e = launch_slab_factor(h->geom, h->strips[jj], h->d_pool[0], sc, h->d_status, h->stream,
                                             &h->timer);
     }
     const cudaError_t idle = cudaStreamSynchronize(h->stream);   // no launch of a failed sequence outlives the scratch
@@ -1170,7 +1165,7 @@ helm_status run_precond_slabs(helm_dd* h, const double2* in, double2* out, int B
     auto solve = [&](int j, const SweepStep& sp, int slot) -> cudaError_t {
         SlabWork wk{rbuf, ybuf[slot], sp.prev >= 0 ? ybuf[slot ^ 1] : nullptr,
                     (const char*)h->d_slab_sxz + h->slab_sxz_off[j] * (int64_t)h->esize, h->ct_sz,
-                    h->slab_cy.data(), ld, B, h->d_slab_scratch, (unsigned*)bf.counters, h->d_status};
+                    ld, B, h->d_slab_scratch, (unsigned*)bf.counters, h->d_status};
         const StripDev* pst = sp.prev >= 0 ? &h->strips[sp.prev] : nullptr;
         if (mixed) return launch_slab_solve<float2>(h->geom, h->strips[j], pst, sp, wk, h->d_pool[0], h->stream, &h->timer);
         return launch_slab_solve<double2>(h->geom, h->strips[j], pst, sp, wk, h->d_pool[0], h->stream, &h->timer);
@@ -1647,7 +1642,7 @@ helm_status run_local_solves(helm_dd* h, const double2* F, double2* Ut, int B, c
         for (int j = 0; j < J; ++j) {
             const SweepStep sp = step_of(j);
             SlabWork wk{rbuf, ybuf, nullptr, (const char*)h->d_slab_sxz + h->slab_sxz_off[j] * (int64_t)h->esize,
-                        h->ct_sz, h->slab_cy.data(), ld, B, h->d_slab_scratch, (unsigned*)bf.counters, h->d_status};
+                        h->ct_sz, ld, B, h->d_slab_scratch, (unsigned*)bf.counters, h->d_status};
             cudaError_t e = mixed ? launch_slab_solve<float2>(h->geom, h->strips[j], nullptr, sp, wk, h->d_pool[0],
                                                               h->stream, &h->timer)
                                   : launch_slab_solve<double2>(h->geom, h->strips[j], nullptr, sp, wk, h->d_pool[0],

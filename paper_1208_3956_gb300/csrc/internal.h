@@ -79,8 +79,8 @@ struct TimedLaunch {
 };
 
 // ---- factor.cu
-// shared memory of a factor kernel with nbuf W x W buffers (3, or 4 for the
-// level-2 separator system)
+// shared memory, static and dynamic, of a factor kernel with nbuf W x W buffers (3, or 4 for
+// the level-2 separator system)
 constexpr size_t kFactorSmemMax = 227 * 1024;
 size_t factor_smem_bytes(int Wmax, size_t esize, int nbuf);
 // pool: Sinv, GT, GB (per grid row), Rinv, E, F, GT2, GB2, P2L, P2U (per separator)
@@ -181,7 +181,6 @@ struct SlabWork {
     const void* pybuf;
     const void* sxz;          // this strip's s_x(c) s_z(z), working precision, n entries
     int64_t ct_sz;            // offset of s_z(z) in Geom::ct
-    const double2* cy_host;   // host: -alpha_y(y_{k-1/2}) / h^2, k = 0 .. Ny
     int ld;                   // row stride of rbuf / ybuf / pybuf (>= every strip's n)
     int B;
     void* scratch;            // slab_sweep_scratch bytes: the strip solve's step vectors and partial sums
@@ -189,9 +188,8 @@ struct SlabWork {
     int* status;              // error word (7 = a bounded wait gave up)
 };
 size_t slab_sweep_scratch(int nmax, size_t esize);
-// Factor blocks X_k = S_k^{-1} of strip st into pool + st.fac (tile layout of slab_ops.cuh,
-// st.bs elements per block), k = 0 .. Ny-1.
-template <typename C>
+// Complex128 factor blocks X_k = S_k^{-1} of strip st into pool + st.fac (tile layout of
+// slab_ops.cuh, st.bs elements per block), k = 0 .. Ny-1.
 cudaError_t launch_slab_factor(const Geom& g, const StripDev& st, void* pool, const SlabScratch& sc, int* status,
                                cudaStream_t s, KernelTimer* tm);
 // slab_tc.cu: the blocks X_k = S_k^{-1}, k = 0 .. Ny-1, of up to 8 strips (16 chains) side by
@@ -226,8 +224,8 @@ cudaError_t launch_stencil(const Geom& g, const double2* u, const double2* f, do
                            cudaStream_t s, KernelTimer* tm);
 cudaError_t launch_copy_cols(const double2* src, double2* dst, int B, int Nx, int Ny, int Nz, int xlo, int xhi,
                              cudaStream_t s, KernelTimer* tm);
-// (coef, if given: -h[b][i] where act[b] != 0, else 0)
-// partial[b][i][blk] for h[b][i] = sum_n conj(V_i[b][n]) w[b][n]; V_i at V + i*vstride
+// out[b][i] = h[b][i] = sum_n conj(V_i[b][n]) w[b][n], V_i at V + i*vstride, summed from
+// partial[b][i][blk] in a fixed order; coef, if given: -h[b][i] where act[b] != 0, else 0
 cudaError_t launch_multidot(const double2* V, int64_t vstride, const double2* w, int nv, int B, int64_t N,
                             double2* partial, int nblk, double2* out, cudaStream_t s, KernelTimer* tm,
                             double2* coef = nullptr, const double* act = nullptr);

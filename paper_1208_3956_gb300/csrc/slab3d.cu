@@ -299,7 +299,7 @@ struct SlabSweepArgs {
     const C* X;          // block 0 of the strip in the tile layout (slab_ops.cuh); block k at X + k * bs
     int64_t bs;
     int n, Ny;
-    int nq, kc, ncta, epc, slots;
+    int nq, kc, epc, slots;
     const C* rhs;        // [B][Ny][ld] right-hand sides
     C* Y;                // [B][Ny][ld] solution
     int ld, B;           // row stride of rhs / Y; right-hand sides of this launch (<= NB)
@@ -320,6 +320,7 @@ constexpr int kProdWarps = 8, kSumThreads = 96;
 constexpr int kSweepThreads = 32 * kProdWarps + 2 * kSumThreads + 32;
 constexpr int kSlotBytes = 16 * 1024;   // a ring slot: 16 (complex64) or 8 columns of 128 rows
 constexpr int kMaxSlots = 16;
+constexpr size_t kSlabSmemMax = 227 * 1024;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mb_init(uint64_t* m, uint32_t count) {
@@ -694,9 +695,9 @@ int grid_for(int64_t work, int threads) {
 }  // namespace
 
 // ------------------------------------------------------------------ host
-template <typename C>
 cudaError_t launch_slab_factor(const Geom& g, const StripDev& st, void* pool, const SlabScratch& sc, int* status,
                                cudaStream_t s, KernelTimer* tm) {
+    using C = double2;
     const int n = st.W * g.Nz;
     if (n > kGjThreads * kGjRowsPerThread) return cudaErrorInvalidValue;
     int dev = 0, nsm = 0, occ = 0;
@@ -771,12 +772,11 @@ struct SlabKernel {
 };
 template <typename C, int NB>
 static bool slab_kernel(const SlabGrid& gr, SlabKernel& k) {
-    constexpr size_t kSmemMax = 227 * 1024;
     const size_t fixed = slab_sweep_fixed<C, NB>(gr.kc);
-    if (gr.epc > SlabTile<NB>::kMaxEpc || fixed + 4 * kSlotBytes > kSmemMax) return false;
+    if (gr.epc > SlabTile<NB>::kMaxEpc || fixed + 4 * kSlotBytes > kSlabSmemMax) return false;
     k.fn = (const void*)k_slab_sweep<C, NB>;
     k.nb = NB;
-    k.slots = (int)std::min<size_t>(kMaxSlots, (kSmemMax - fixed) / kSlotBytes);
+    k.slots = (int)std::min<size_t>(kMaxSlots, (kSlabSmemMax - fixed) / kSlotBytes);
     k.smem = fixed + (size_t)k.slots * kSlotBytes;
     return true;
 }
@@ -804,20 +804,16 @@ static cudaError_t sm_count(int& nsm) {
     return e;
 }
 // Shared-memory limits of every variant on the current device (this also loads them).
-template <typename C>
 static cudaError_t slab_kernel_attrs() {
-    cudaError_t e = cudaFuncSetAttribute(k_gj_invert<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGjCacheMax);
-    auto set = [&](const void* fn) {
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaError_t e = cudaSuccess;
+    auto set = [&](const void* fn, size_t bytes) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     };
-    set((const void*)k_slab_sweep<C, 1>);
-    if constexpr (std::is_same<C, float2>::value) {
-        set((const void*)k_slab_sweep<C, 4>);
-        set((const void*)k_slab_sweep<C, 8>);
-        set((const void*)k_slab_sweep<C, 16>);
-    } else {
-        set((const void*)k_slab_sweep<C, 2>);
-    }
+    for (const void* fn : {(const void*)k_slab_sweep<float2, 1>, (const void*)k_slab_sweep<float2, 4>,
+                           (const void*)k_slab_sweep<float2, 8>, (const void*)k_slab_sweep<float2, 16>,
+                           (const void*)k_slab_sweep<double2, 1>, (const void*)k_slab_sweep<double2, 2>})
+        set(fn, kSlabSmemMax);
+    set((const void*)k_gj_invert<double2>, kGjCacheMax);
     return e;
 }
 
@@ -863,7 +859,6 @@ cudaError_t launch_slab_solve(const Geom& g, const StripDev& st, const StripDev*
         A.Ny = Ny;
         A.nq = gr.nq;
         A.kc = gr.kc;
-        A.ncta = gr.ncta;
         A.epc = gr.epc;
         A.slots = kr.slots;
         A.rhs = Rb + (int64_t)b0 * Ny * ld;
@@ -901,8 +896,7 @@ cudaError_t launch_slab_out(const Geom& g, const StripDev& st, int dir, const vo
 // Loads this file's kernels onto the current device and sets their shared-memory limits there.
 cudaError_t preload_slab_kernels() {
     cudaFuncAttributes fa;
-    cudaError_t e = slab_kernel_attrs<float2>();
-    if (e == cudaSuccess) e = slab_kernel_attrs<double2>();
+    cudaError_t e = slab_kernel_attrs();
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_rhs<float2>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_rhs<double2>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_out<float2>);
@@ -911,8 +905,6 @@ cudaError_t preload_slab_kernels() {
 }
 
 #define HELM_SLAB_INST(C)                                                                                       \
-    template cudaError_t launch_slab_factor<C>(const Geom&, const StripDev&, void*, const SlabScratch&, int*,   \
-                                               cudaStream_t, KernelTimer*);                                    \
     template cudaError_t launch_slab_solve<C>(const Geom&, const StripDev&, const StripDev*, const SweepStep&, \
                                               const SlabWork&, const void*, cudaStream_t, KernelTimer*);       \
     template cudaError_t launch_slab_out<C>(const Geom&, const StripDev&, int, const void*, int, double2*,     \

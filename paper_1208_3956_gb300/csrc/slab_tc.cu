@@ -1,9 +1,10 @@
 // Tensor-core factorisation of the dense 3-D strip blocks (Section 2.3, Algorithm 1 on
 // strips whose block row is a whole x-z slab), complex64.
 //
-// Every block X_k = S_k^{-1}, S_k = D_k - C_k X_{k-1} C_k (n x n, n = W N_z), is inverted
-// by blocked Gauss-Jordan elimination with partial pivoting, the J strips of the grid side
-// by side and in each strip the two chains toward the middle row (slab3d.cu).  Pivot rows are not exchanged: a row that has served as the pivot of a column is
+// Every block X_k = S_k^{-1} (n x n, n = W N_z; S_k = D_k less C_k X_{k-1} C_k above the middle row,
+// C_{k+1} X_{k+1} C_{k+1} below it and both at it, slab3d.cu) is inverted by blocked Gauss-Jordan
+// elimination with partial pivoting, up to 8 strips of the grid side by side and in each strip
+// the two chains toward the middle row.  Pivot rows are not exchanged: a row that has served as the pivot of a column is
 // marked (kstep) and left out of later pivot searches.  The columns go in panels of kTcBig,
 // each made of sub-panels of kTcSub:
 //
