@@ -43,8 +43,9 @@ def builtin_chunks(Ny: int) -> int:
 
 def candidates(Ny: int, dim: int = 2, nrhs: int = 1) -> list:
     """(P, G) pairs around the built-in choice: P at 0.7 .. 1.3 of it, G around sqrt(P-1).
-    Panels of more than 4 right-hand sides run as several tiles of P+1 CTAs, which favour
-    fewer, longer chunks: their P range reaches down to a sixth of the built-in one."""
+    Panels of more than 4 right-hand sides run as several tiles of P+1 CTAs (4 right-hand sides
+    to a tile in complex64, one in complex128 as long as that takes few rounds of the SMs), which
+    favour fewer, longer chunks: their P range reaches down to a sixth of the built-in one."""
     if dim == 3:
         return [(0, 0)]
     P0 = builtin_chunks(Ny)

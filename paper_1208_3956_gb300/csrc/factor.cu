@@ -703,7 +703,7 @@ static cudaError_t launch_factor_ni(const Geom& g, int Wmax, void* const* pool, 
     // A chunk's chain of inversions and products leaves most issue slots empty (barriers, shared
     // memory), so a third CTA per SM helps once the grid has more than two for each: complex64
     // 3 x 3 tiles fit in its 80 registers without spills.  Factor of 1023 x 1023 30.5 -> 27.5 ms,
-    // 511 x 511 9.6 -> 9.1; four CTAs (64 registers, spills) 27.9 and 9.35.  Smaller grids keep
+    // 511 x 511 9.6 -> 9.0; four CTAs (64 registers, spills) 27.9 and 9.35.  Smaller grids keep
     // the registers (127 x 127: 2.75 ms against 2.79), and so does complex128, bound by the FP64
     // pipe.
     constexpr int kMinB = sizeof(C) == 8 && NI == 3 ? 3 : 0;

@@ -288,10 +288,12 @@ __global__ void k_slab_rhs(Geom g, StripDev st, SweepStep sp, StripDev pst, cons
 // sides, the right-hand sides in two), their sums meet in shared memory once per step.
 // What bounds it: with one right-hand side the chain's latency under the stream's load (tile
 // 7.4k cycles, the rest of a step about 12k, half of it hidden by the other chain); with 16
-// the shared-memory reads and FP32 FMAs of the tile.  One application of P on the 63^3 grid
+// instruction issue (54 %, the FMA pipe 40 %, shared memory 30 % on a 39^3 grid) and the barriers
+// that end a step; in complex128 the FP64 pipe (83 % with two on 33 x 37 x 29).  One application of P on the 63^3 grid
 // (8 strips, blocks of 1659-1817, 15 strip solves; top-down elimination with whole rows per
 // CTA and tiles of 4 right-hand sides before): 16.4 -> 11.3 ms with one right-hand side (3.2
-// -> 4.7 TB/s of blocks), 127 -> 28.3 ms with 16.
+// -> 4.7 TB/s of blocks), 127 -> 28.3 ms with 16.  Complex128 on 33 x 37 x 29 (blocks of 779 and
+// 820): 21.3 -> 6.5, 60.1 -> 9.7 and 59.9 -> 19.2 ms with 1, 2 and 4.
 // Every wait is bounded: on time-out the kernel records 7 in the status word, waits (bounded)
 // for its copies in flight and returns.
 template <typename C>
@@ -781,8 +783,8 @@ static bool slab_kernel(const SlabGrid& gr, SlabKernel& k) {
     return true;
 }
 // For `left` remaining right-hand sides: the widest useful tile that fits (a tile streams every
-// block once whatever its width).  Complex128 takes two at most: its products are bound by the
-// FP64 pipe, not by the stream.
+// block once whatever its width).  Complex128 takes two at most: the FP64 pipe is 83 % busy
+// then and DRAM 9 %, so a wider tile would stream less and take as long.
 template <typename C>
 static SlabKernel pick_slab_kernel(const SlabGrid& gr, int left) {
     SlabKernel k;

@@ -16,8 +16,9 @@
 //   * the last chunk CTA of a separator group to finish (atomic arrival
 //     counter per group, no waiting) solves the group's separators with the
 //     level-2 separators held at zero (twisted chain z_i = a_i - E_i z_outer,
-//     x_i = z_i - F_i x_inner) and adds the group's parts of the level-2
-//     right-hand sides; the last group to finish solves the level-2 system.
+//     x_i = z_i - F_i x_inner);
+//   * with separator groups one more CTA per tile solves the level-2 system, once every
+//     chunk has added its contributions to the level-2 right-hand sides.
 // k_sweep_output (work items: chunks x strips x RHS tiles, grid-stride)
 //   final separator values (grouped separators: x_q = y_q - GT2_q x2_above -
 //   GB2_q x2_below), then x_k = y_k - GT_p(k) x_{p-1} - GB_p(k) x_p on the output
@@ -1756,8 +1757,9 @@ cudaError_t launch_outputs(const OutArgs& O, void* const* pool, cudaStream_t s, 
     if (O.nstrip <= 0) return cudaSuccess;
     TimedLaunch t(tm, "sweep_output", s);
     const C *GT = (const C*)pool[1], *GB = (const C*)pool[2], *GT2 = (const C*)pool[6], *GB2 = (const C*)pool[7];
-    // several right-hand sides in complex64: the spike rows once for all of them (complex128 is
-    // bound by the FP64 pipe, which a padded group of four right-hand sides would waste)
+    // several right-hand sides in complex64: the spike rows once for all of them.  In complex128 the
+    // strip solves beside these passes hold the FP64 pipe, and a padded group of four right-hand
+    // sides would take more of it
     const bool panel = O.Bt > 1 && sizeof(C) == sizeof(float2);
     const int bt = panel ? kPanelOut : O.Bt;
     const int nitem = O.g.P * O.nstrip * ((O.B + bt - 1) / bt);
