@@ -448,10 +448,11 @@ cudaError_t launch_add(double2* dst, const double2* src, int64_t n, cudaStream_t
     return cudaGetLastError();
 }
 
-// Loads this file's module onto the current device.
-cudaError_t preload_field_kernels() {
+cudaError_t preload_field_kernels(int dim) {
     cudaFuncAttributes fa;
-    return cudaFuncGetAttributes(&fa, k_copy_cols);
+    cudaError_t e = cudaFuncGetAttributes(&fa, k_copy_cols);
+    if (e != cudaSuccess) return e;
+    return dim == 3 ? cudaFuncGetAttributes(&fa, k_stencil<true>) : cudaFuncGetAttributes(&fa, k_stencil<false>);
 }
 
 }  // namespace helm

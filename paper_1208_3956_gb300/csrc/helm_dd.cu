@@ -409,14 +409,16 @@ helm_status ensure_device(helm_dd* h) {
         CK(h, cudaEventCreateWithFlags(&h->ev_main, cudaEventDisableTiming));
         CK(h, cudaEventCreateWithFlags(&h->ev_side, cudaEventDisableTiming));
     }
-    // Everything a later call launches is loaded now, where allocation is expected:
-    // the no-allocation scratch array (its address cached per device) and the
-    // modules of the sweep, slab and grid kernels.
+    // What a preconditioner call of this handle needs is loaded now, where allocation is
+    // expected: the no-allocation scratch array (its address cached per device) and its kernels.
     CK(h, noalloc_scratch(&h->noalloc_base));
-    CK(h, preload_sweep_kernels());
-    CK(h, preload_slab_kernels());
-    CK(h, preload_tc_kernels());
-    CK(h, preload_field_kernels());
+    if (h->dim == 2) {
+        CK(h, preload_sweep_kernels(h->esize));
+    } else {
+        CK(h, preload_slab_kernels(h->esize));
+        if (h->prec == HELM_PREC_MIXED) CK(h, preload_tc_kernels());
+    }
+    CK(h, preload_field_kernels(h->dim));
     const int64_t nint = (int64_t)h->c.size();
     CK(h, cudaMalloc(&h->d_c, nint * sizeof(double)));
     CK(h, cudaMalloc(&h->d_k2, nvol(h) * sizeof(double)));

@@ -207,14 +207,17 @@ template <typename C>
 cudaError_t launch_slab_out(const Geom& g, const StripDev& st, int dir, const void* ybuf, int ld, double2* dst,
                             const double2* base, int B, cudaStream_t s, KernelTimer* tm);
 
-// Load each file's kernels onto the current device (lazy loading would otherwise load them,
-// and take their memory, at the first launch inside some later call) and set the
-// shared-memory limits of those that need more than 48 KB; once per handle, at its first
-// device use.
-cudaError_t preload_sweep_kernels();
-cudaError_t preload_slab_kernels();
+// Load onto the current device the kernels that an application of the preconditioner launches
+// with elements of esize bytes (2-D: sweep.cu; 3-D: slab3d.cu; field.cu), and set the shared-memory
+// limits of the kernels that need more than 48 KB (the 3-D factorisation's too).  Lazy loading
+// would load them, and take their memory, at the first launch inside some later call.  Once per
+// handle, at its first device use, and no others than the handle's: more kernels on the device
+// make the short ones slower (1023 x 1023, complex64, one P: 4.149 ms, 4.167 with both precisions
+// and the 3-D kernels loaded).
+cudaError_t preload_sweep_kernels(size_t esize);
+cudaError_t preload_slab_kernels(size_t esize);
 cudaError_t preload_tc_kernels();
-cudaError_t preload_field_kernels();
+cudaError_t preload_field_kernels(int dim);
 
 // ---- field.cu: FP64 grid kernels
 cudaError_t launch_k2(const double* c_int, double* k2, int dim, int nx, int ny, int nz, int w, double omega,

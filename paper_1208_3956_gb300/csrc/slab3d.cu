@@ -805,20 +805,6 @@ static cudaError_t sm_count(int& nsm) {
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     return e;
 }
-// Shared-memory limits of every variant on the current device (this also loads them).
-static cudaError_t slab_kernel_attrs() {
-    cudaError_t e = cudaSuccess;
-    auto set = [&](const void* fn, size_t bytes) {
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    };
-    for (const void* fn : {(const void*)k_slab_sweep<float2, 1>, (const void*)k_slab_sweep<float2, 4>,
-                           (const void*)k_slab_sweep<float2, 8>, (const void*)k_slab_sweep<float2, 16>,
-                           (const void*)k_slab_sweep<double2, 1>, (const void*)k_slab_sweep<double2, 2>})
-        set(fn, kSlabSmemMax);
-    set((const void*)k_gj_invert<double2>, kGjCacheMax);
-    return e;
-}
-
 // Z and P of the strip solve, for strips of up to nmax unknowns.
 size_t slab_sweep_scratch(int nmax, size_t esize) {
     int nsm = 0;
@@ -895,14 +881,25 @@ cudaError_t launch_slab_out(const Geom& g, const StripDev& st, int dir, const vo
     return cudaGetLastError();
 }
 
-// Loads this file's kernels onto the current device and sets their shared-memory limits there.
-cudaError_t preload_slab_kernels() {
+cudaError_t preload_slab_kernels(size_t esize) {
     cudaFuncAttributes fa;
-    cudaError_t e = slab_kernel_attrs();
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_rhs<float2>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_rhs<double2>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_out<float2>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_out<double2>);
+    cudaError_t e = cudaSuccess;
+    auto limit = [&](const void* fn, size_t bytes) {   // (this also loads the kernel)
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    if (esize == sizeof(float2)) {
+        for (const void* fn : {(const void*)k_slab_sweep<float2, 1>, (const void*)k_slab_sweep<float2, 4>,
+                               (const void*)k_slab_sweep<float2, 8>, (const void*)k_slab_sweep<float2, 16>})
+            limit(fn, kSlabSmemMax);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_rhs<float2>);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_out<float2>);
+    } else {
+        limit((const void*)k_slab_sweep<double2, 1>, kSlabSmemMax);
+        limit((const void*)k_slab_sweep<double2, 2>, kSlabSmemMax);
+        limit((const void*)k_gj_invert<double2>, kGjCacheMax);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_rhs<double2>);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_slab_out<double2>);
+    }
     return e;
 }
 

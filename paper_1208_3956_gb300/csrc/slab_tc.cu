@@ -575,7 +575,6 @@ __global__ void __launch_bounds__(256) k_tc_store(const __grid_constant__ TcArgs
     S.X[slab_at(n, r, c)] = (pc < n && q >= 0 && q < n) ? S.M[(int64_t)pc * S.ldm + q] : make_float2(0.f, 0.f);
 }
 
-// Loads the update kernels onto the current device and sets their shared-memory limit there.
 cudaError_t preload_tc_kernels() {
     cudaError_t e = cudaFuncSetAttribute(k_tc_update<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcUpdSmem);
     if (e == cudaSuccess)

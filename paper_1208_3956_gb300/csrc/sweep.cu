@@ -1679,7 +1679,7 @@ int strip_solve_tile(const Geom& g, const StripDev& st, int zrows, size_t esize,
                                    : planned_tile<double2>(st, zrows, tile_width<double2>(B, ctas, sh));
 }
 
-// Shared-memory limit of every strip-solve instantiation (this also loads the module).
+// Shared-memory limit of every strip-solve instantiation (this also loads them).
 template <typename C>
 static cudaError_t chunk_kernel_attrs() {
     cudaError_t e = cudaSuccess;
@@ -1693,13 +1693,13 @@ static cudaError_t chunk_kernel_attrs() {
     return e;
 }
 
-cudaError_t preload_sweep_kernels() {
-    cudaError_t e = chunk_kernel_attrs<float2>();
-    if (e == cudaSuccess) e = chunk_kernel_attrs<double2>();
+cudaError_t preload_sweep_kernels(size_t esize) {
+    const bool c64 = esize == sizeof(float2);
     cudaFuncAttributes fa;
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_sweep_output<float2>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_sweep_output<double2>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_sweep_output_panel<float2>);
+    cudaError_t e = c64 ? chunk_kernel_attrs<float2>() : chunk_kernel_attrs<double2>();
+    if (e == cudaSuccess)
+        e = c64 ? cudaFuncGetAttributes(&fa, k_sweep_output<float2>) : cudaFuncGetAttributes(&fa, k_sweep_output<double2>);
+    if (e == cudaSuccess && c64) e = cudaFuncGetAttributes(&fa, k_sweep_output_panel<float2>);
     return e;
 }
 
