@@ -719,9 +719,10 @@ __global__ void __launch_bounds__(BT == 1 ? 288 : chunk_threads(4 * NJ, BT)) k_s
     const bool upw = kPanel && w >= 2 * nrb;                    // panel: a warp of the up chain
     const int bp = kPanel ? (w / nrb) & 1 : 0;                  // panel: pair of right-hand sides
     const int ob = 2 * bp + g;                                  // panel: the right-hand side this lane finishes
-    // panel: the warp's pair has a right-hand side (a ragged tile's absent pair multiplies nothing; its
-    // products cost a complex128 tile of 1 or 2 as much FP64 pipe as the present ones)
-    const bool pairon = compute && 2 * bp < nb;
+    // panel: the warp multiplies.  In complex128 a ragged tile's absent pair does not: its products
+    // would take as much of the FP64 pipe as the present ones (255 x 255 concurrent, 6 right-hand sides:
+    // 7.9 -> 7.3 ms); complex64 is not bound by them, and the test costs a full tile 1 % on small grids
+    const bool pairon = compute && (sizeof(C) == sizeof(float2) || 2 * bp < nb);
     const bool rowok = compute && row < W;
     const bool own = kPanel && rowok && ob < nb;
     const int rc = imin(row, W - 1);
