@@ -208,7 +208,7 @@ helm_status helm_dd_apply_precond(helm_dd* h, const double* in, double* out, int
  * device memory, programs near the memory limit where a late workspace
  * allocation could fail, and latency-critical loops where cudaMalloc/cudaFree
  * would stall the device.  The work buffers come from one 64 MiB file-scope
- * device array.  The array (and every kernel module the call launches) is
+ * device array.  The array (and every kernel the call launches) is
  * loaded onto a device, and its 64 MiB taken, when a handle first uses that
  * device (in helm_dd_factor, with the handle's other device memory); its
  * device address is looked up there too, once per device with that device

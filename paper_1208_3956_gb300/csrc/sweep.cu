@@ -721,7 +721,8 @@ __global__ void __launch_bounds__(BT == 1 ? 288 : chunk_threads(4 * NJ, BT)) k_s
     const int ob = 2 * bp + g;                                  // panel: the right-hand side this lane finishes
     // panel: the warp multiplies.  In complex128 a ragged tile's absent pair does not: its products
     // would take as much of the FP64 pipe as the present ones (255 x 255 concurrent, 6 right-hand sides:
-    // 7.9 -> 7.3 ms); complex64 is not bound by them, and the test costs a full tile 1 % on small grids
+    // 7.9 -> 7.3 ms); complex64 is not bound by them, and the test costs a full tile 1 % (255 x 511, J = 32,
+    // 4 right-hand sides: 2.106 ms without it, 2.134 with)
     const bool pairon = compute && (sizeof(C) == sizeof(float2) || 2 * bp < nb);
     const bool rowok = compute && row < W;
     const bool own = kPanel && rowok && ob < nb;
